@@ -24,6 +24,7 @@
 #include <string>
 
 #include "../../include/cslbm.h"
+#include "lattice_const.h"
 
 cslbm_status cslbm_record_error(cslbm_status s, const char* msg);
 
@@ -52,7 +53,7 @@ constexpr int NF = 6;
 struct Lat {
     int n[2], lo[2], hi[2];
     long long N;
-    double omega, kvisc, theta, fext[2];
+    cslbm::Cst omega, kvisc, theta, fext[2];
     const double* face[4];  // [2][n other] contravariant face velocity, or null
 };
 

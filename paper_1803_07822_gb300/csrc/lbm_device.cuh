@@ -20,6 +20,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lattice_const.h"
+
 namespace cslbm {
 
 constexpr int Q = 19;
@@ -74,10 +76,10 @@ struct Lat {
     int n[3];
     int bclo[3], bchi[3];
     long long N;
-    double omega;      // 1/tau
-    double kvisc;      // 1 - 1/(2 tau)
-    double theta;
-    double fext[3];
+    Cst omega;         // 1/tau
+    Cst kvisc;         // 1 - 1/(2 tau)
+    Cst theta;
+    Cst fext[3];
     const double* face[6];  // contravariant boundary velocity [3][face nodes] or null
 };
 
