@@ -25,6 +25,7 @@
 
 #include "../../include/cslbm.h"
 #include "lattice_const.h"
+#include "widen.cuh"
 
 cslbm_status cslbm_record_error(cslbm_status s, const char* msg);
 
@@ -844,8 +845,10 @@ __global__ void __launch_bounds__(TB) k2_transform(Lat L, const R* __restrict__ 
     }
 }
 
+// (five blocks per SM: at the registers the face path would take, three fit,
+// and the loads' latency showed)
 template <class R>
-__global__ void __launch_bounds__(TB) k2_readout(Lat L, const R* __restrict__ P, const R* __restrict__ Fc,
+__global__ void __launch_bounds__(TB, sizeof(R) == 8 ? 2 : 5) k2_readout(const __grid_constant__ Lat L, const R* __restrict__ P, const R* __restrict__ Fc,
                                                  const R* __restrict__ G, const double* __restrict__ J4,
                                                  double* __restrict__ rho_out, double* __restrict__ u_out,
                                                  int cartesian)
@@ -853,12 +856,28 @@ __global__ void __launch_bounds__(TB) k2_readout(Lat L, const R* __restrict__ P,
     const long long v = blockIdx.x * (long long)TB + threadIdx.x;
     if (v >= L.N) return;
     const long long N = L.N;
-    const int x = (int)(v % L.n[0]), y = (int)(v / L.n[0]);
+    // 32-bit division where the lattice allows it (a 64-bit one is about a hundred instructions)
+    const int y = N < (1LL << 32) ? (int)((unsigned)v / (unsigned)L.n[0]) : (int)(v / L.n[0]);
+    const int x = (int)(v - (long long)y * L.n[0]);
     R h[Q], Fo[NF], rho, j[2], Pi[3];
     node_state<R>(L, P, Fc, G, x, y, h, Fo);
     moments_h<R>(h, G[v], Fo, rho, j, Pi);
-    const double u0 = double(j[0]) / double(rho), u1 = double(j[1]) / double(rho);
-    rho_out[v] = double(rho);
+    // FP32: one reciprocal for both components (two divisions and three
+    // conversions kept the FP64 pipe busy for 186 us at 4096 x 1024, where
+    // the bytes take 64; now 105 us); FP64 or unusual values: the division
+    double u0, u1, r;
+    bool odd = sizeof(R) == 8;
+    if constexpr (sizeof(R) == 4) {
+        const double ir = cslbm::recip64(rho, r, odd);
+        u0 = cslbm::widen(j[0], odd) * ir;
+        u1 = cslbm::widen(j[1], odd) * ir;
+    }
+    if (odd) {
+        r = double(rho);
+        u0 = double(j[0]) / r;
+        u1 = double(j[1]) / r;
+    }
+    rho_out[v] = r;
     if (cartesian) {
         u_out[v] = J4[v] * u0 + J4[N + v] * u1;
         u_out[N + v] = J4[2 * N + v] * u0 + J4[3 * N + v] * u1;

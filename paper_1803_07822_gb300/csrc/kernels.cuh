@@ -11,6 +11,7 @@
 #include "lbm_device.cuh"
 #include "fp_convert.h"
 #include "make_lat.h"
+#include "widen.cuh"
 
 namespace cslbm {
 
@@ -18,12 +19,13 @@ constexpr int TPB = 256;
 
 inline unsigned nblocks(long long n) { return (unsigned)((n + TPB - 1) / TPB); }
 
+// (32-bit arithmetic: a context holds fewer than 2^32 / 25 nodes)
 __device__ __forceinline__ void node_coords(const Lat& L, long long v, int& x, int& y, int& z)
 {
-    x = (int)(v % L.n[0]);
-    long long r = v / L.n[0];
-    y = (int)(r % L.n[1]);
-    z = (int)(r / L.n[1]);
+    const unsigned vu = (unsigned)v, n0 = L.n[0], n1 = L.n[1], row = vu / n0, zr = row / n1;
+    x = (int)(vu - row * n0);
+    y = (int)(row - zr * n1);
+    z = (int)zr;
 }
 
 // ---------------------------------------------------------------------------
@@ -625,8 +627,94 @@ __global__ void __launch_bounds__(TPB) k_transform_interp(Lat L, S* __restrict__
 // ---------------------------------------------------------------------------
 // readout and reductions
 // ---------------------------------------------------------------------------
+// rho and j of a node; face nodes (the boundary rule) out of line, few take it
 template <class S, class R>
-__global__ void __launch_bounds__(TPB) k_readout(Lat L, const S* __restrict__ P, const R* __restrict__ hist,
+__device__ __noinline__ Mom4<R> face_density(const Lat& L, const S* __restrict__ P, const R* __restrict__ hist,
+                                             const R* __restrict__ geo, int x, int y, int z)
+{
+    const long long v = nidx(L, x, y, z);
+    NodeMoments<S, R> M;
+    node_moments<S, R>(L, P, hist, geo, x, y, z, v, geo[v], M);
+    return Mom4<R>{M.j[0], M.j[1], M.j[2], M.rho};
+}
+
+// u = j / rho and, with J, v = J u, by FP64 division: the values the quick
+// forms below do not cover
+struct Vec3 {
+    double x, y, z;
+};
+template <class R>
+__device__ __noinline__ Vec3 velocity_any(R rho, R j0, R j1, R j2, const R* __restrict__ J, long long N)
+{
+    const double u[3] = {double(j0) / double(rho), double(j1) / double(rho), double(j2) / double(rho)};
+    if (!J) return Vec3{u[0], u[1], u[2]};
+    auto row = [&](int a) {
+        return double(J[(a * 3 + 0) * N]) * u[0] + double(J[(a * 3 + 1) * N]) * u[1] + double(J[(a * 3 + 2) * N]) * u[2];
+    };
+    return Vec3{row(0), row(1), row(2)};
+}
+
+// The readout of one node.  It is bound by the FP64 pipe unless FP64
+// instructions are few: with three divisions and 13 conversions per node
+// 256^3 took 1,398 us, where the node's 188 bytes take 463; with 16 FP64
+// instructions and four blocks per SM (64 registers) it takes 635.  One reciprocal of rho serves all components: 1/rho from an
+// FP32 estimate and two Newton steps (error below 2^-52), u = j/rho with one
+// residual correction, v = (J j)/rho, the products of FP32 values exact.
+__device__ __forceinline__ double density_velocity(float rho, const float j[3], const float* __restrict__ J,
+                                                   long long N, double out[3])
+{
+    bool odd = false;
+    double r, jd[3];
+    const double ir = recip64(rho, r, odd);
+#pragma unroll
+    for (int a = 0; a < 3; a++) jd[a] = widen(j[a], odd);
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        if (J) {
+            const double s = fma(widen(J[(a * 3 + 2) * N], odd), jd[2],
+                                 fma(widen(J[(a * 3 + 1) * N], odd), jd[1], widen(J[(a * 3) * N], odd) * jd[0]));
+            out[a] = s * ir;
+        } else {
+            const double q = jd[a] * ir;
+            out[a] = fma(fma(-q, r, jd[a]), ir, q);
+        }
+    }
+    if (odd) {
+        const Vec3 w = velocity_any<float>(rho, j[0], j[1], j[2], J, N);
+        out[0] = w.x;
+        out[1] = w.y;
+        out[2] = w.z;
+        return double(rho);
+    }
+    return r;
+}
+// FP64 storage: one division for the three components, each corrected by its residual
+__device__ __forceinline__ double density_velocity(double rho, const double j[3], const double* __restrict__ J,
+                                                   long long N, double out[3])
+{
+    auto plain = [](double v) { return fabs(v) < 0x1p500 && (fabs(v) > 0x1p-500 || v == 0.0); };
+    if (!(rho > 0x1p-400 && rho < 0x1p400 && plain(j[0]) && plain(j[1]) && plain(j[2]))) {
+        const Vec3 w = velocity_any<double>(rho, j[0], j[1], j[2], J, N);
+        out[0] = w.x;
+        out[1] = w.y;
+        out[2] = w.z;
+        return rho;
+    }
+    const double ir = 1.0 / rho;
+    double u[3];
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const double q = j[a] * ir;
+        u[a] = fma(fma(-q, rho, j[a]), ir, q);
+    }
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+        out[a] = J ? J[(a * 3 + 0) * N] * u[0] + J[(a * 3 + 1) * N] * u[1] + J[(a * 3 + 2) * N] * u[2] : u[a];
+    return rho;
+}
+
+template <class S, class R>
+__global__ void __launch_bounds__(TPB, 4) k_readout(const __grid_constant__ Lat L, const S* __restrict__ P, const R* __restrict__ hist,
                                                  const R* __restrict__ geo, const R* __restrict__ J,
                                                  double* __restrict__ rho_out, double* __restrict__ u_out,
                                                  long long stride, long long v0, long long cnt, int cartesian)
@@ -636,21 +724,29 @@ __global__ void __launch_bounds__(TPB) k_readout(Lat L, const S* __restrict__ P,
     long long v = v0 + t;
     int x, y, z;
     node_coords(L, v, x, y, z);
-    NodeMoments<S, R> M;
-    node_moments<S, R>(L, P, hist, geo, x, y, z, v, geo[v], M);
-    double u[3];
+    R rho, j[3];
+    if (on_boundary(L, x, y, z)) {
+        const Mom4<R> m = face_density<S, R>(L, P, hist, geo, x, y, z);
+        rho = m.w;
+        j[0] = m.x;
+        j[1] = m.y;
+        j[2] = m.z;
+    } else {
+        // (the same sums as node_moments)
+        R s[Q], m0, m1[3], m2[6];
+        const R sg = geo[v];
+        gather_raw<S, R>(L, P, x, y, z, s);
+        sums(s, m0, m1, m2);
+        rho = sg * (R(1) + m0) + R(0.5) * hist[v];
 #pragma unroll
-    for (int a = 0; a < 3; a++) u[a] = double(M.j[a]) / double(M.rho);
-    if (rho_out) rho_out[t] = double(M.rho);
+        for (int a = 0; a < 3; a++) j[a] = sg * m1[a] + R(0.5) * hist[(1 + a) * L.N + v];
+    }
+    double u[3];
+    const double r = density_velocity(rho, j, cartesian ? J + v : nullptr, L.N, u);
+    if (rho_out) rho_out[t] = r;
     if (u_out) {
 #pragma unroll
-        for (int a = 0; a < 3; a++) {
-            double s = u[a];
-            if (cartesian)
-                s = double(J[(a * 3 + 0) * L.N + v]) * u[0] + double(J[(a * 3 + 1) * L.N + v]) * u[1] +
-                    double(J[(a * 3 + 2) * L.N + v]) * u[2];
-            u_out[a * stride + t] = s;
-        }
+        for (int a = 0; a < 3; a++) u_out[a * stride + t] = u[a];
     }
 }
 
