@@ -68,8 +68,11 @@ def step_pass(n, storage, step_kernel, axis2_periodic=False):
     sb = {"fp32": 4, "fp16": 2, "bf16": 2}.get(storage)
     rows = (step_kernel in ("auto", "rows") and sb is not None and n[0] <= 256 and n[0] % 4 == 0
             and (n[0] * sb) % 16 == 0 and n[0] * n[1] * n[2] >= 256)
-    if rows and step_kernel == "auto" and not axis2_periodic:
-        return "fused"
+    if rows and step_kernel == "auto":
+        tr = min(256 // n[0], n[1])
+        if tr * n[0] != 256 or n[0] * n[1] * n[2] < (3 << 20 if sb == 4 else 12 << 20):
+            return "flat"
+        return "rows" if axis2_periodic else "fused"
     return "rows" if rows else "flat"
 
 

@@ -75,10 +75,11 @@ typedef struct {
  * n[0] <= 256, n[0] a multiple of 4, n[0] * bytes per stored population a
  * multiple of 16 and at least 256 nodes.  Its fused form also forms the
  * momentum field in the same (cooperative) launch; it needs axis 2 to be
- * non-periodic.  AUTO takes the fused row pass, else the row pass, else the
- * flat gather pass; ROWS the row pass (momentum field in a kernel of its
- * own), else the flat pass; FLAT always the flat pass.  All give the same
- * results up to rounding. */
+ * non-periodic.  AUTO takes the fused row pass, else the row pass, where they
+ * apply and pay (256 a multiple of n[0]; at least 3,145,728 nodes in FP32,
+ * 12,582,912 in FP16 / BF16), else the flat gather pass; ROWS the row pass
+ * (momentum field in a kernel of its own) where it applies, else the flat
+ * pass; FLAT always the flat pass.  All give the same results up to rounding. */
 typedef enum { CSLBM_STEP_AUTO = 0, CSLBM_STEP_FLAT = 1, CSLBM_STEP_ROWS = 2 } cslbm_step_kernel;
 
 typedef struct cslbm_ctx cslbm_ctx;

@@ -92,6 +92,45 @@ __device__ __forceinline__ void grid_barrier(unsigned* count, int* err)
     __syncthreads();
 }
 
+// the step of a node on a face, out of line
+__device__ __noinline__ void step_face(const Lat& L, const float* __restrict__ Pin, float* __restrict__ Pout,
+                                       const float* __restrict__ hin, float* __restrict__ hout,
+                                       const float* __restrict__ geo, const Mom4<float>* __restrict__ jf, int x, int y,
+                                       int z)
+{
+    step_boundary_body<float, float>(L, Pin, Pout, hin, hout, geo, jf, x, y, z);
+}
+
+__device__ __forceinline__ void step_node(const Lat& L, const float* __restrict__ Pin, float* __restrict__ Pout,
+                                          const float* __restrict__ hin, float* __restrict__ hout,
+                                          const float* __restrict__ geo, const Mom4<float>* __restrict__ jf, int x,
+                                          int y, int z, unsigned v)
+{
+    const unsigned N = (unsigned)L.N;
+    if (on_boundary(L, x, y, z)) {
+        step_face(L, Pin, Pout, hin, hout, geo, jf, x, y, z);
+        return;
+    }
+    const Nbr src = nbr_index(L, x, y, z, -1);
+    float s[Q];
+#pragma unroll
+    for (int l = 0; l < Q; l++)
+        s[l] = __ldg(Pin + (unsigned)pslot(l) * N + nbr_off(src, cvec(l, 0), cvec(l, 1), cvec(l, 2)));
+    GeoT<float> G;
+    HistT<float> Hp;
+    load_geo_hist(geo, hin, v, N, G, Hp);
+    float d[9][3];
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        const int l = 2 * k + 1, cx = cvec(l, 0), cy = cvec(l, 1), cz = cvec(l, 2);
+        const Mom4<float> p = jf[nbr_off(src, -cx, -cy, -cz)], m = jf[nbr_off(src, cx, cy, cz)];
+        d[k][0] = p.x - m.x;
+        d[k][1] = p.y - m.y;
+        d[k][2] = p.z - m.z;
+    }
+    step_core<float, float>(L, s, G, Hp, d, Pout, hout, v, N);
+}
+
 // One persistent launch per LBM step of every channel (see the top of the
 // file).  first[c] = first work item of channel c (items of `item` nodes),
 // first[nchan] = all items; q[0], q[1] the momentum and step queues and
@@ -125,7 +164,7 @@ __global__ void __launch_bounds__(TB) k_batch_persistent(const Chan* __restrict_
                 if (phase == 0)
                     momentum_node<float, float>(C.L, C.P[pi], C.H[hi], C.G, C.jf, x, y, z, v);
                 else
-                    step_node<float, float>(C.L, C.P[pi], C.P[pi ^ 1], C.H[hi], C.H[hi ^ 1], C.G, C.jf, x, y, z, v);
+                    step_node(C.L, C.P[pi], C.P[pi ^ 1], C.H[hi], C.H[hi ^ 1], C.G, C.jf, x, y, z, v);
             }
         }
         if (phase == 0) grid_barrier(&q[2], err);

@@ -5,15 +5,27 @@
 // pass forms rho u of every node (one float4 per node, a field small enough
 // to stay in L2); the second pass steps every node independently: pull
 // gather, moments, stress, gradient from the neighbours' rho u, forcing
-// moments, collision, store.  No barriers and no shared memory, so the SMs
-// run at the occupancy the registers allow; the price over the one-pass
-// ideal is one extra read of the populations per step.
+// moments, collision, store.  No barriers, so the SMs run at the occupancy
+// the registers allow; the price over the one-pass ideal is one extra read
+// of the populations per step (about 430 B per node against 332).
 //
-// Nodes on a non-periodic face take one generic out-of-line path (boundary
-// rule, ghost extrapolation of the stencil); every other node has all its
-// pull sources and stencil sites inside the domain after periodic wrapping.
+// What bounds them (GB300, FP32, 128 x 256 x 128): the momentum pass the
+// memory, 63 us for 418 MB, the measured copy rate; the step pass the latency
+// of its loads at 16 warps per SM, 288 us for 1,433 MB (0.73 of the copy
+// rate, 41 % of issue slots).  The split into short chains is what made it
+// so: geometry and history travel to shared memory asynchronously while the
+// populations and the stencil load (64x128x64: 76.6 -> 46 us per step, 91 x
+// 77 x 93: 94 -> 60, 256^3: 1,717 -> 1,334 with the following), face nodes
+// run in blocks of their own ahead of the others instead of on a slow branch
+// of every warp, rho u of a face node needs no boundary rule, blocks shrink
+// until every SM has four (16 x 32 x 16: 22.6 -> 13.3 us per step, FP64 106
+// -> 51), and each kernel's blocks come up while the previous one drains.
+// Measured without effect: five blocks per SM, blocks of 64 or 160 nodes,
+// descending order, evict-first stores; an L2 prefetch one wave ahead costs
+// 10 to 30 %.
 #pragma once
 
+#include "fast_div.h"
 #include "step_math.cuh"
 
 namespace cslbm {
@@ -44,79 +56,86 @@ __device__ __forceinline__ unsigned nbr_off(const Nbr& p, int cx, int cy, int cz
     return p.zs[cz + 1] + p.ys[cy + 1] + p.xs[cx + 1];
 }
 
-// rho u of a boundary node from the boundary rule
-template <class S, class R>
-__device__ __noinline__ void momentum_boundary(const Lat& L, const S* __restrict__ P, const R* __restrict__ hist,
-                                               const R* __restrict__ geo, int x, int y, int z, Mom4<R>* jf)
-{
-    R s[Q];
-    boundary_pops<S, R>(L, P, hist, geo, x, y, z, s);
-    PairSums<R> Ps;
-    pair_sums(s, Ps);
-    R m1[3];
-    first_moment(Ps, m1);
-    const long long v = nidx(L, x, y, z);
-    const R sg = geo[v];
-    Mom4<R> j;
-    j.x = fmad(sg, m1[0], R(0.5) * hist[1 * L.N + v]);
-    j.y = fmad(sg, m1[1], R(0.5) * hist[2 * L.N + v]);
-    j.z = fmad(sg, m1[2], R(0.5) * hist[3 * L.N + v]);
-    j.w = R(0);
-    jf[v] = j;
-}
-
-// launch shape of both passes: blocks of 256 consecutive nodes of a plane
-// (blockIdx.x), one grid row per plane (blockIdx.y)
-constexpr int TB = 256;
-
-__device__ __forceinline__ bool flat_node(const Lat& L, int& x, int& y, int& z, unsigned& v)
-{
-    const unsigned n01 = (unsigned)L.n[0] * L.n[1];
-    const unsigned r = blockIdx.x * (unsigned)TB + threadIdx.x;
-    if (r >= n01) return false;
-    y = (int)(r / (unsigned)L.n[0]);
-    x = (int)(r - (unsigned)y * L.n[0]);
-    z = blockIdx.y;
-    v = (unsigned)z * n01 + r;
-    return true;
-}
-
-// rho u of one node into jf[v] (pull gather; boundary rule on face nodes)
+// rho u of one node into jf[v].  A face node's follows from its inner node
+// without the boundary rule's populations: a wall or inflow node takes
+// rho_i u_w (the first moment of f^eq(rho_i, u_w) plus that of the inner
+// node's non-equilibrium part, which vanishes), an outflow node takes j_i.
+// So every node makes the same gather, a face node at its inner node.
 template <class S, class R>
 __device__ __forceinline__ void momentum_node(const Lat& L, const S* __restrict__ P, const R* __restrict__ hist,
                                               const R* __restrict__ geo, Mom4<R>* __restrict__ jf, int x, int y,
                                               int z, unsigned v)
 {
     const unsigned N = (unsigned)L.N;
-    if (on_boundary(L, x, y, z)) {
-        momentum_boundary<S, R>(L, P, hist, geo, x, y, z, jf);
-        return;
-    }
-    const Nbr src = nbr_index(L, x, y, z, -1);
+    const bool face = on_boundary(L, x, y, z);
+    const int r[3] = {x, y, z};
+    int in[3] = {x, y, z}, axis = 0, side = 0, bc = BC_OUTFLOW;
+    if (face) bc = classify(L, r, axis, side, in);
+    const Nbr src = nbr_index(L, in[0], in[1], in[2], -1);
     R s[Q];
 #pragma unroll
     for (int l = 0; l < Q; l++)
         s[l] = R(Store<S>::ld(P + (unsigned)pslot(l) * N + nbr_off(src, cvec(l, 0), cvec(l, 1), cvec(l, 2))));
+    const unsigned vi = nbr_off(src, 0, 0, 0);
+    const R sg = __ldg(geo + vi);
+    Mom4<R> j;
+    j.x = __ldg(hist + 1 * N + vi);
+    j.y = __ldg(hist + 2 * N + vi);
+    j.z = __ldg(hist + 3 * N + vi);
+    j.w = R(0);
     PairSums<R> Ps;
     pair_sums(s, Ps);
     R m1[3];
     first_moment(Ps, m1);
-    const R sg = __ldg(geo + v);
-    Mom4<R> j;
-    j.x = fmad(sg, m1[0], R(0.5) * __ldg(hist + 1 * N + v));
-    j.y = fmad(sg, m1[1], R(0.5) * __ldg(hist + 2 * N + v));
-    j.z = fmad(sg, m1[2], R(0.5) * __ldg(hist + 3 * N + v));
-    j.w = R(0);
+    j.x = fmad(sg, m1[0], R(0.5) * j.x);
+    j.y = fmad(sg, m1[1], R(0.5) * j.y);
+    j.z = fmad(sg, m1[2], R(0.5) * j.z);
+    if (bc != BC_OUTFLOW) {
+        R m0 = s[0];
+#pragma unroll
+        for (int k = 0; k < 9; k++) m0 += Ps.p[k];
+        const R rho = fmad(sg, m0 + R(1), R(0.5) * __ldg(hist + vi));
+        R u[3];
+        face_velocity(L, axis, side, r, u);
+        j.x = rho * u[0];
+        j.y = rho * u[1];
+        j.z = rho * u[2];
+    }
     jf[v] = j;
 }
 
+// Both passes run over consecutive nodes of the lattice, one thread each, in
+// blocks of FB threads or fewer (flat_block).
+constexpr int FB = 128;
+
+struct Plane {
+    Div n0, n01;
+};
+__device__ __forceinline__ void flat_coords(const Lat& L, const Plane& pl, unsigned v, int& x, int& y, int& z)
+{
+    const unsigned n0 = L.n[0], zu = div_by(v, pl.n01), r = v - zu * (n0 * (unsigned)L.n[1]), yu = div_by(r, pl.n0);
+    x = (int)(r - yu * n0);
+    y = (int)yu;
+    z = (int)zu;
+}
+
+// The kernels of a step follow one another with programmatic launches: the
+// next kernel's blocks come up while the last blocks of this one still run
+// and wait here for its completion before they touch memory.
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
 template <class S, class R>
-__global__ void __launch_bounds__(TB) k_momentum_flat(Lat L, const S* __restrict__ P, const R* __restrict__ hist,
+__global__ void __launch_bounds__(FB) k_momentum_flat(const __grid_constant__ Lat L, const __grid_constant__ Plane pl,
+                                                      const S* __restrict__ P, const R* __restrict__ hist,
                                                       const R* __restrict__ geo, Mom4<R>* __restrict__ jf)
 {
+    const unsigned v = blockIdx.x * blockDim.x + threadIdx.x;
     int x, y, z;
-    unsigned v;
-    if (!flat_node(L, x, y, z, v)) return;
+    flat_coords(L, pl, v, x, y, z);
+    wait_previous();
+    launch_next();
+    if (v >= (unsigned)L.N) return;
     momentum_node<S, R>(L, P, hist, geo, jf, x, y, z, v);
 }
 
@@ -315,60 +334,6 @@ __device__ __forceinline__ void step_boundary_body(const Lat& L, const S* __rest
     step_core<S, R>(L, s, G, Hp, d, Pout, hout, v, N);
 }
 
-// out of line where face nodes share a kernel with interior nodes
-template <class S, class R>
-__device__ __noinline__ void step_boundary(const Lat& L, const S* __restrict__ Pin, S* __restrict__ Pout,
-                                           const R* __restrict__ hin, R* __restrict__ hout, const R* __restrict__ geo,
-                                           const Mom4<R>* __restrict__ jf, int x, int y, int z)
-{
-    step_boundary_body<S, R>(L, Pin, Pout, hin, hout, geo, jf, x, y, z);
-}
-
-// the step of one node: pull gather, moments, gradient from the rho u field,
-// forcing, collision, store (the boundary rule and ghost stencil out of line
-// on face nodes)
-template <class S, class R>
-__device__ __forceinline__ void step_node(const Lat& L, const S* __restrict__ Pin, S* __restrict__ Pout,
-                                          const R* __restrict__ hin, R* __restrict__ hout, const R* __restrict__ geo,
-                                          const Mom4<R>* __restrict__ jf, int x, int y, int z, unsigned v)
-{
-    const unsigned N = (unsigned)L.N;
-    if (on_boundary(L, x, y, z)) {
-        step_boundary<S, R>(L, Pin, Pout, hin, hout, geo, jf, x, y, z);
-        return;
-    }
-    const Nbr src = nbr_index(L, x, y, z, -1);
-    R s[Q];
-#pragma unroll
-    for (int l = 0; l < Q; l++)
-        s[l] = R(Store<S>::ld(Pin + (unsigned)pslot(l) * N + nbr_off(src, cvec(l, 0), cvec(l, 1), cvec(l, 2))));
-    GeoT<R> G;
-    HistT<R> Hp;
-    load_geo_hist(geo, hin, v, N, G, Hp);
-    const Nbr nb = nbr_index(L, x, y, z, +1);  // sites x + c
-    R d[9][3];
-#pragma unroll
-    for (int k = 0; k < 9; k++) {
-        const int l = 2 * k + 1, cx = cvec(l, 0), cy = cvec(l, 1), cz = cvec(l, 2);
-        const Mom4<R> p = jf[nbr_off(nb, cx, cy, cz)], m = jf[nbr_off(nb, -cx, -cy, -cz)];
-        d[k][0] = p.x - m.x;
-        d[k][1] = p.y - m.y;
-        d[k][2] = p.z - m.z;
-    }
-    step_core<S, R>(L, s, G, Hp, d, Pout, hout, v, N);
-}
-
-template <class S, class R>
-__global__ void __launch_bounds__(TB, 2) k_step_flat(Lat L, const S* __restrict__ Pin, S* __restrict__ Pout,
-                                                     const R* __restrict__ hin, R* __restrict__ hout,
-                                                     const R* __restrict__ geo, const Mom4<R>* __restrict__ jf)
-{
-    int x, y, z;
-    unsigned v;
-    if (!flat_node(L, x, y, z, v)) return;
-    step_node<S, R>(L, Pin, Pout, hin, hout, geo, jf, x, y, z, v);
-}
-
 // The nodes on non-periodic faces as up to six boxes without overlap: the
 // faces of axis 2 whole, those of axis 1 without the axis-2 face nodes, those
 // of axis 0 without the face nodes of axes 1 and 2.
@@ -408,18 +373,12 @@ inline FaceList face_list(const cslbm_ctx* c)
     return f;
 }
 
-// one step of the face nodes only (the interior comes from the row-staged pass)
-template <class S, class R>
-__global__ void __launch_bounds__(128) k_step_faces(const __grid_constant__ Lat L, const __grid_constant__ FaceList f,
-                                                    const S* __restrict__ Pin, S* __restrict__ Pout,
-                                                    const R* __restrict__ hin, R* __restrict__ hout,
-                                                    const R* __restrict__ geo, const Mom4<R>* __restrict__ jf)
+// node i of the list; false past its end.  (Selects over the six segments: an
+// index of f by a runtime value would copy it to local memory; face nodes
+// number fewer than 2^31.)
+__device__ __forceinline__ bool face_coords(const FaceList& f, int i, int& x, int& y, int& z)
 {
-    // face nodes number fewer than 2^31 (the lattice's nodes do)
-    const int i = blockIdx.x * 128 + threadIdx.x;
-    if (i >= (int)f.start[f.nseg]) return;
-    // segment of node i, by selects over the six (no indexing of f by a
-    // runtime value, which would copy it to local memory)
+    if (i >= (int)f.start[f.nseg]) return false;
     int lo0 = 0, lo1 = 0, lo2 = 0, len0 = 1, len1 = 1, st = 0;
 #pragma unroll
     for (int k = 0; k < 6; k++)
@@ -432,9 +391,21 @@ __global__ void __launch_bounds__(128) k_step_faces(const __grid_constant__ Lat 
             st = (int)f.start[k];
         }
     const int r = i - st, q = r / len0;
-    const int x = lo0 + (r - q * len0);
-    const int y = lo1 + q % len1;
-    const int z = lo2 + q / len1;
+    x = lo0 + (r - q * len0);
+    y = lo1 + q % len1;
+    z = lo2 + q / len1;
+    return true;
+}
+
+// one step of the face nodes only (the interior comes from the row-staged pass)
+template <class S, class R>
+__global__ void __launch_bounds__(128) k_step_faces(const __grid_constant__ Lat L, const __grid_constant__ FaceList f,
+                                                    const S* __restrict__ Pin, S* __restrict__ Pout,
+                                                    const R* __restrict__ hin, R* __restrict__ hout,
+                                                    const R* __restrict__ geo, const Mom4<R>* __restrict__ jf)
+{
+    int x, y, z;
+    if (!face_coords(f, blockIdx.x * 128 + threadIdx.x, x, y, z)) return;
     step_boundary_body<S, R>(L, Pin, Pout, hin, hout, geo, jf, x, y, z);
 }
 
@@ -450,15 +421,139 @@ int launch_faces(const cslbm_ctx* c, const Lat& L, const S* Pin, S* Pout, const 
     return 1;
 }
 
-inline dim3 flat_grid(const cslbm_ctx* c)
+// asynchronous copy of one value into shared memory
+__device__ __forceinline__ void copy_async(float* dst, const float* src)
 {
-    return dim3((unsigned)(((long long)c->n[0] * c->n[1] + TB - 1) / TB), c->n[2]);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copy_async(double* dst, const double* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copies_landed() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+// The step of an interior node.  The 35 values of its geometry and history
+// travel to shared memory (sm[k * FB], the thread's own column: no barrier)
+// while the populations and the rho u stencil, which the arithmetic needs
+// first, are loaded into registers, so that all of the node's reads are in
+// flight at once.
+template <class S, class R>
+__device__ __forceinline__ void step_interior(const Lat& L, const S* __restrict__ Pin, S* __restrict__ Pout,
+                                              const R* __restrict__ hin, R* __restrict__ hout,
+                                              const R* __restrict__ geo, const Mom4<R>* __restrict__ jf, int x, int y,
+                                              int z, unsigned v, R* sm)
+{
+    const unsigned N = (unsigned)L.N;
+    {
+        const R* g = geo + v;
+        const R* h = hin + v;
+#pragma unroll
+        for (int k = 0; k < NGEO; k++) copy_async(sm + k * FB, g + (size_t)k * N);
+#pragma unroll
+        for (int k = 0; k < NHIST; k++) copy_async(sm + (NGEO + k) * FB, h + (size_t)k * N);
+    }
+    const Nbr src = nbr_index(L, x, y, z, -1);
+    R s[Q];
+#pragma unroll
+    for (int l = 0; l < Q; l++)
+        s[l] = R(Store<S>::ld(Pin + (unsigned)pslot(l) * N + nbr_off(src, cvec(l, 0), cvec(l, 1), cvec(l, 2))));
+    R d[9][3];
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        // site x + c is the pull source of -c
+        const int l = 2 * k + 1, cx = cvec(l, 0), cy = cvec(l, 1), cz = cvec(l, 2);
+        const Mom4<R> p = jf[nbr_off(src, -cx, -cy, -cz)], m = jf[nbr_off(src, cx, cy, cz)];
+        d[k][0] = p.x - m.x;
+        d[k][1] = p.y - m.y;
+        d[k][2] = p.z - m.z;
+    }
+    copies_landed();
+    GeoT<R> G;
+    HistT<R> Hp;
+    G.sg = sm[0];
+    G.isg = recip(G.sg);
+#pragma unroll
+    for (int a = 0; a < 6; a++) G.gi[a] = sm[(1 + a) * FB];
+#pragma unroll
+    for (int a = 0; a < 18; a++) G.gam[a] = sm[(7 + a) * FB];
+#pragma unroll
+    for (int k = 0; k < 3; k++) G.gc[k] = (G.gam[0 * 6 + s6(k, 0)] + G.gam[1 * 6 + s6(k, 1)]) + G.gam[2 * 6 + s6(k, 2)];
+    Hp.A = sm[NGEO * FB];
+#pragma unroll
+    for (int a = 0; a < 3; a++) Hp.B[a] = sm[(NGEO + 1 + a) * FB];
+#pragma unroll
+    for (int a = 0; a < 6; a++) Hp.C[a] = sm[(NGEO + 4 + a) * FB];
+    step_core<S, R>(L, s, G, Hp, d, Pout, hout, v, N);
+}
+
+// The step of every node: the first nfb blocks take the face nodes (the
+// longest chains of loads, so they start first), the others the nodes of the
+// planes between non-periodic faces of axis 2, v = v0 ..
+template <class S, class R>
+__global__ void __launch_bounds__(FB, sizeof(R) == 8 ? 3 : 4)
+    k_step_flat(const __grid_constant__ Lat L, const __grid_constant__ Plane pl, const __grid_constant__ FaceList f,
+                unsigned nfb, unsigned v0, unsigned v1, const S* __restrict__ Pin, S* __restrict__ Pout,
+                const R* __restrict__ hin, R* __restrict__ hout, const R* __restrict__ geo,
+                const Mom4<R>* __restrict__ jf)
+{
+    __shared__ R sm[(NGEO + NHIST) * FB];
+    int x, y, z;
+    if (blockIdx.x < nfb) {
+        const bool ok = face_coords(f, (int)(blockIdx.x * blockDim.x + threadIdx.x), x, y, z);
+        wait_previous();
+        launch_next();
+        if (ok) step_boundary_body<S, R>(L, Pin, Pout, hin, hout, geo, jf, x, y, z);
+        return;
+    }
+    const unsigned v = v0 + (blockIdx.x - nfb) * blockDim.x + threadIdx.x;
+    flat_coords(L, pl, v, x, y, z);
+    wait_previous();
+    launch_next();
+    if (v >= v1 || on_boundary(L, x, y, z)) return;
+    step_interior<S, R>(L, Pin, Pout, hin, hout, geo, jf, x, y, z, v, sm + threadIdx.x);
+}
+
+// threads per block: FB, fewer where that would leave multiprocessors idle
+inline unsigned flat_block(const cslbm_ctx* c)
+{
+    unsigned tb = FB;
+    while (tb > 32 && c->N < (long long)tb * 4 * c->n_sm) tb /= 2;
+    return tb;
+}
+
+inline Plane make_plane(const Lat& L)
+{
+    Plane p;
+    p.n0 = make_div((unsigned)L.n[0]);
+    p.n01 = make_div((unsigned)L.n[0] * (unsigned)L.n[1]);
+    return p;
+}
+
+// a kernel whose blocks may come up before the previous one has ended (it
+// waits for that itself)
+template <class... A>
+inline void launch_after(void (*kernel)(A...), unsigned grid, unsigned block, cudaStream_t stream, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 template <class S, class R>
 void launch_momentum(const cslbm_ctx* c, const Lat& L, const S* P, const R* hin, const R* geo)
 {
-    k_momentum_flat<S, R><<<flat_grid(c), TB, 0, c->stream>>>(L, P, hin, geo, (Mom4<R>*)c->jf);
+    const unsigned tb = flat_block(c);
+    launch_after(k_momentum_flat<S, R>, (unsigned)((c->N + tb - 1) / tb), tb, c->stream, L, make_plane(L), P, hin, geo,
+                 (Mom4<R>*)c->jf);
 }
 
 // one time step: momentum pass, then the step pass
@@ -466,8 +561,13 @@ template <class S, class R>
 void launch_flat_step(const cslbm_ctx* c, const Lat& L, const S* Pin, S* Pout, const R* hin, R* hout, const R* geo)
 {
     launch_momentum<S, R>(c, L, Pin, hin, geo);
-    k_step_flat<S, R><<<flat_grid(c), TB, 0, c->stream>>>(L, Pin, Pout, hin, hout, geo,
-                                                                         (const Mom4<R>*)c->jf);
+    const unsigned tb = flat_block(c);
+    const FaceList f = face_list(c);
+    const unsigned nfb = (unsigned)((f.start[f.nseg] + tb - 1) / tb), n01 = (unsigned)c->n[0] * c->n[1];
+    const bool zper = c->p.bc_lo[2] == CSLBM_PERIODIC;
+    const unsigned v0 = zper ? 0 : n01, v1 = zper ? (unsigned)c->N : (unsigned)c->N - n01;
+    launch_after(k_step_flat<S, R>, nfb + (v1 - v0 + tb - 1) / tb, tb, c->stream, L, make_plane(L), f, nfb, v0, v1, Pin,
+                 Pout, hin, hout, geo, (const Mom4<R>*)c->jf);
 }
 
 }  // namespace cslbm

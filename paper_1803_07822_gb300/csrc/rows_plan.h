@@ -62,6 +62,19 @@ inline bool make_plan(const int n[3], bool yper, bool zper, int s_bytes, int max
     return (long long)smem_bytes(pl) <= max_smem;
 }
 
+// Whether the row passes beat the gather pass where they apply.  They need
+// full tiles (TR n0 = NT: all compute threads busy, grouped copies; 192-node
+// rows: 742 us fused, 574 gather at 192^3 FP32) and a lattice well beyond L2,
+// where one read of the populations less counts: measured in us per step,
+// fused / gather, FP32 128^3 192 / 175, 256x256x48 264 / 271, 256x256x96
+// 463 / 515, 256^3 1,138 / 1,334; FP16 256x256x96 444 / 431, 256x256x192
+// 818 / 838.  Hence 3.1 million nodes for FP32, 12.6 million for 16 bits.
+inline bool pays(const Plan& pl, const int n[3], int s_bytes)
+{
+    const long long N = (long long)n[0] * n[1] * n[2];
+    return pl.TR * n[0] == NT && N >= (s_bytes == 4 ? 3LL << 20 : 12LL << 20);
+}
+
 // smem layout of the fused pass after the two step stages: the momentum
 // stage (populations, sqrt(g), A and B; off_sg and off_h4 relative to it),
 // two rho u tiles of NT nodes, then ten mbarriers; false when it does not fit
