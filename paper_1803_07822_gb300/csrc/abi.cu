@@ -406,10 +406,12 @@ cslbm_status cslbm_update_metric_interp(cslbm_ctx* c, const double* g6, const do
     if (!scratch || scratch_bytes < 20 * (size_t)c->N * c->r_bytes) return fail(CSLBM_ENOMEM, "scratch too small");
     for (const void* q : {(const void*)g6, (const void*)dg18, (const void*)Jnew9, (const void*)psi3, (const void*)scratch})
         if (!is_device_memory(q)) return fail(CSLBM_EINVAL, "every array of update_metric_interp is device memory");
-    if (cslbm_status s = run_metric(c, g6, dg18, 1, 1 - c->gc, false)) return s;
-    c->ops->transform_interp(c, Jnew9, psi3, scratch);
+    int* bad = (int*)(c->scratch + 32);
+    if (!c->metric_check_pending) CUDA_TRY(cudaMemsetAsync(bad, 0, sizeof(int), c->stream));
+    c->ops->transform_interp(c, g6, dg18, Jnew9, psi3, scratch, bad);
     c->launches += 2;
     LAUNCH_CHECK("interpolating transform kernels");
+    c->metric_check_pending = 1;
     if (cslbm_status s = store_jacobian(c, Jnew9, c->N, 0, c->N)) return s;
     c->pc ^= 1;
     c->hc ^= 1;

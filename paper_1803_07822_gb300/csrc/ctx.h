@@ -100,10 +100,11 @@ struct cslbm_ops {
     void (*chart_change)(const cslbm_ctx*, const double* g6, const double* dg18, const double* Jnew, int* bad);
     void (*chart_change_mixed)(const cslbm_ctx*, const double* g6, const float* dg18, const float* Jnew, int* bad);
     // chart change with interpolation: the transformation inputs of every node
-    // into scratch [20][N] (precision R), then every node of P[1-pc],H[1-hc]
-    // from them at psi3 [3][N] (old lattice coordinates) with G[1-gc]; J (old)
-    // is read, not written
-    void (*transform_interp)(const cslbm_ctx*, const double* Jnew, const double* psi3, void* scratch);
+    // into scratch [20][N] (precision R), then G[1-gc] from g6/dg18 and every
+    // node of P[1-pc],H[1-hc] from the inputs at psi3 [3][N] (old lattice
+    // coordinates); J (old) is read, not written; *bad as above
+    void (*transform_interp)(const cslbm_ctx*, const double* g6, const double* dg18, const double* Jnew,
+                             const double* psi3, void* scratch, int* bad);
     // rho, u (or v) of nodes [v0, v0+cnt) into out arrays with the given stride
     void (*readout)(const cslbm_ctx*, double* rho, double* u3, long long stride, long long v0,
                     long long cnt, int cartesian);

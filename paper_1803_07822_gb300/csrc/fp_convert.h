@@ -25,16 +25,17 @@ CSLBM_HD float f64_to_f32_rn(double x)
 {
     uint64_t u;
     memcpy(&u, &x, 8);
-    const uint32_t hi = (uint32_t)(u >> 32), lo = (uint32_t)u;
-    const uint32_t sign = hi & 0x80000000u;
-    const int e = (int)((hi >> 20) & 0x7ffu) - 1023 + 127;  // binary32 biased exponent
-    const uint32_t m = ((hi & 0xfffffu) << 3) | (lo >> 29);  // the 23 kept fraction bits
-    const uint32_t rest = lo & 0x1fffffffu;                  // the 29 dropped ones
-    // a carry out of the fraction moves into the exponent, as rounding wants
-    uint32_t r = ((uint32_t)(e > 0 ? e : 0) << 23) + m;
-    r += (rest > 0x10000000u || (rest == 0x10000000u && (m & 1u))) ? 1u : 0u;
-    if (e <= 0) r = 0u;
-    if (e >= 255 || r >= 0x7f800000u) r = 0x7f800000u;
+    const uint32_t sign = (uint32_t)(u >> 32) & 0x80000000u;
+    // half an ulp less one, plus the last kept bit: the carry out of the 29
+    // dropped bits rounds to nearest with ties to even, and a carry out of
+    // the fraction moves into the exponent, as rounding wants
+    u += 0x0fffffffu + ((uint32_t)(u >> 29) & 1u);
+    // high word without its sign, its exponent rebiased: from 2^20 to 255 2^20
+    // exclusive for results in the normal range
+    const int32_t h = (int32_t)((uint32_t)(u >> 32) & 0x7fffffffu) - (896 << 20);
+    uint32_t r = ((uint32_t)h << 3) | ((uint32_t)u >> 29);
+    if (h < (1 << 20)) r = 0u;
+    if (h >= (255 << 20)) r = 0x7f800000u;
     r |= sign;
     float f;
     memcpy(&f, &r, 4);

@@ -426,19 +426,6 @@ __device__ __forceinline__ void dphi_of(const Cm (&n)[9], const Cm (&o)[9], R (&
         }
 }
 
-// the same from FP64 Jacobians, rounded to Cm first
-template <class Cm, class R>
-__device__ __forceinline__ void dphi(const double (&Jn)[9], const double (&Jo)[9], R (&Dp)[3][3])
-{
-    Cm n[9], o[9];
-#pragma unroll
-    for (int k = 0; k < 9; k++) {
-        n[k] = to_real<Cm>(Jn[k]);
-        o[k] = to_real<Cm>(Jo[k]);
-    }
-    dphi_of<Cm, R>(n, o, Dp);
-}
-
 // the f-moments and history of a node in the form the transformation takes:
 // out = {rho, j[3], M2[6], A, B[3], Cs[6]}
 template <class S, class R>
@@ -542,8 +529,9 @@ __global__ void __launch_bounds__(TPB, 3) k_chart(Lat L, const S* __restrict__ P
 
 // Chart change with interpolation, pass 1: the transformation inputs of every
 // old node into mf [20][N]
+// (four blocks per SM: 37 -> 32 us on 256 x 256 x 16 FP32)
 template <class S, class R>
-__global__ void __launch_bounds__(TPB) k_moment_fields(Lat L, const S* __restrict__ Pin, const R* __restrict__ hin,
+__global__ void __launch_bounds__(TPB, sizeof(R) == 8 ? 2 : 4) k_moment_fields(const __grid_constant__ Lat L, const S* __restrict__ Pin, const R* __restrict__ hin,
                                                        const R* __restrict__ geo_old, R* __restrict__ mf, int literal)
 {
     const long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -556,13 +544,21 @@ __global__ void __launch_bounds__(TPB) k_moment_fields(Lat L, const S* __restric
     for (int k = 0; k < 20; k++) mf[k * L.N + v] = in[k];
 }
 
+// p modulo n into [0, n], as fmod(p, n) (+ n when negative) has it
+static __device__ __noinline__ double wrap_far(double p, int n)
+{
+    p = fmod(p, (double)n);
+    return p < 0.0 ? p + n : p;
+}
 // trilinear corners of the point p (old lattice coordinates) along one axis:
-// a periodic axis wraps, a non-periodic one clamps p to [0, n - 1]
+// a periodic axis wraps, a non-periodic one clamps p to [0, n - 1].  Points
+// less than one period outside wrap by one addition (fmod is a loop of FP64
+// instructions; both give the same value: p - n is exact for n <= p < 2n).
 __device__ __forceinline__ void interp_axis(double p, int n, bool per, int& i0, int& i1, double& t)
 {
+    const double dn = (double)n;
     if (per) {
-        p = fmod(p, (double)n);
-        if (p < 0.0) p += n;
+        if (!(p >= 0.0 && p < dn)) p = p < 0.0 && p > -dn ? p + dn : (p >= dn && p < 2.0 * dn ? p - dn : wrap_far(p, n));
     } else {
         p = fmin(fmax(p, 0.0), (double)(n - 1));
     }
@@ -573,55 +569,143 @@ __device__ __forceinline__ void interp_axis(double p, int n, bool per, int& i0, 
     i1 = per ? (i0 + 1 == n ? 0 : i0 + 1) : (i0 + 1 < n ? i0 + 1 : n - 1);
 }
 
-// pass 2: every new node from the fields at psi(x~) = psi3[.][v]
+// The corner weights and the weighted sums of the interpolating transform at
+// the arithmetic's precision.  The old Jacobian is summed in FP64 and rounded
+// to R; the other fields in R with the weights rounded to R.
+template <class R> struct Corners;
+template <> struct Corners<double> {
+    double w[8];
+    __device__ __forceinline__ void set(const double t[3])
+    {
+#pragma unroll
+        for (int c = 0; c < 8; c++)
+            w[c] = (c & 1 ? t[0] : 1.0 - t[0]) * (c & 2 ? t[1] : 1.0 - t[1]) * (c & 4 ? t[2] : 1.0 - t[2]);
+    }
+    __device__ __forceinline__ double weight(int c) const { return w[c]; }
+    __device__ __forceinline__ double wide_sum(const double v[8]) const
+    {
+        double s = 0.0;
+#pragma unroll
+        for (int c = 0; c < 8; c++) s += w[c] * v[c];
+        return s;
+    }
+};
+// FP32: each weight as an unevaluated sum of two FP32 values (48 bits), and
+// the Jacobian's sums by error-free products and additions, so that the
+// result is the FP64 sum rounded to FP32 without FP64 arithmetic.  (72 FP64
+// products and as many conversions per node were 85 % of the FP64 pipe's
+// time and bound the kernel: Ogita, Rump and Oishi's compensated dot product
+// costs about 800 FP32 instructions, an eighth of that time.)
+template <> struct Corners<float> {
+    float h[8], l[8];
+    __device__ __forceinline__ static void split(double v, float& hi, float& lo)
+    {
+        hi = f64_to_f32_rn(v);
+        lo = f64_to_f32_rn(v - f32_to_f64(hi));
+    }
+    __device__ __forceinline__ static void mul(float ah, float al, float bh, float bl, float& h, float& l)
+    {
+        const float p = __fmul_rn(ah, bh);
+        const float e = __fmaf_rn(al, bh, __fmaf_rn(ah, bl, __fmaf_rn(ah, bh, -p)));
+        h = __fadd_rn(p, e);
+        l = __fsub_rn(e, __fsub_rn(h, p));
+    }
+    __device__ __forceinline__ void set(const double t[3])
+    {
+        float ah[3][2], al[3][2];
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            split(1.0 - t[a], ah[a][0], al[a][0]);
+            split(t[a], ah[a][1], al[a][1]);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            float ph, pl;
+            mul(ah[0][q & 1], al[0][q & 1], ah[1][q >> 1], al[1][q >> 1], ph, pl);
+#pragma unroll
+            for (int b = 0; b < 2; b++) mul(ph, pl, ah[2][b], al[2][b], h[q + 4 * b], l[q + 4 * b]);
+        }
+    }
+    __device__ __forceinline__ float weight(int c) const { return h[c]; }
+    __device__ __forceinline__ float wide_sum(const float v[8]) const
+    {
+        float s = 0.0f, rest = 0.0f;
+#pragma unroll
+        for (int c = 0; c < 8; c++) {
+            const float p = __fmul_rn(h[c], v[c]);
+            const float e = __fmaf_rn(l[c], v[c], __fmaf_rn(h[c], v[c], -p));
+            const float n = __fadd_rn(s, p), b = __fsub_rn(n, s);
+            rest = __fadd_rn(rest, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(n, b)), __fsub_rn(p, b)), e));
+            s = n;
+        }
+        return fabsf(rest) <= 3.402823466e38f ? __fadd_rn(s, rest) : s;  // (infinite terms: s itself)
+    }
+};
+
+// pass 2: the new geometry of every node from its metric (as k_metric; *bad
+// set and the geometry left as it was on det g <= 0), then its state from the
+// fields at psi(x~) = psi3[.][v].  One pass for both, so that the metric's
+// FP64 arithmetic runs beside the corner loads (256 x 256 x 16 FP32: 65 + 390
+// us as two kernels, 207 as this one).
 template <class S, class R>
-__global__ void __launch_bounds__(TPB) k_transform_interp(Lat L, S* __restrict__ Pout, R* __restrict__ hout,
-                                                          const R* __restrict__ geo_new, const R* __restrict__ J,
-                                                          const double* __restrict__ Jnew,
-                                                          const double* __restrict__ psi, const R* __restrict__ mf,
-                                                          int literal)
+__global__ void __launch_bounds__(128, sizeof(R) == 8 ? 3 : 5)
+    k_transform_interp(const __grid_constant__ Lat L, S* __restrict__ Pout, R* __restrict__ hout, R* __restrict__ geo_new,
+                       const R* __restrict__ J, const double* __restrict__ g6, const double* __restrict__ dg18,
+                       const double* __restrict__ Jnew, const double* __restrict__ psi, const R* __restrict__ mf,
+                       int literal, int* bad)
 {
-    const long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long v = blockIdx.x * 128LL + threadIdx.x;
     if (v >= L.N) return;
     int x, y, z;
     node_coords(L, v, x, y, z);
-    int c0[3], c1[3];
-    double t[3];
+    unsigned ix[8];
+    Corners<R> W;
+    {
+        int c0[3], c1[3];
+        double t[3];
 #pragma unroll
-    for (int a = 0; a < 3; a++)
-        interp_axis(psi[a * L.N + v], L.n[a], L.bclo[a] == BC_PERIODIC && L.bchi[a] == BC_PERIODIC, c0[a], c1[a],
-                    t[a]);
-    long long ix[8];
-    double w[8];
+        for (int a = 0; a < 3; a++)
+            interp_axis(psi[a * L.N + v], L.n[a], L.bclo[a] == BC_PERIODIC && L.bchi[a] == BC_PERIODIC, c0[a], c1[a],
+                        t[a]);
+        W.set(t);
+        const unsigned n0 = L.n[0], n1 = L.n[1];
 #pragma unroll
-    for (int c = 0; c < 8; c++) {
-        const int b0 = c & 1, b1 = (c >> 1) & 1, b2 = (c >> 2) & 1;
-        ix[c] = nidx(L, b0 ? c1[0] : c0[0], b1 ? c1[1] : c0[1], b2 ? c1[2] : c0[2]);
-        w[c] = (b0 ? t[0] : 1.0 - t[0]) * (b1 ? t[1] : 1.0 - t[1]) * (b2 ? t[2] : 1.0 - t[2]);
-    }
-    double Jo[9], Jn[9];
-#pragma unroll
-    for (int k = 0; k < 9; k++) {
-        double s = 0.0;
-#pragma unroll
-        for (int c = 0; c < 8; c++) s += w[c] * double(J[k * L.N + ix[c]]);
-        Jo[k] = s;
-        Jn[k] = Jnew[k * L.N + v];
+        for (int c = 0; c < 8; c++)
+            ix[c] = ((unsigned)(c & 4 ? c1[2] : c0[2]) * n1 + (unsigned)(c & 2 ? c1[1] : c0[1])) * n0 +
+                    (unsigned)(c & 1 ? c1[0] : c0[0]);
     }
     R Dp[3][3];
-    dphi<R, R>(Jn, Jo, Dp);
+    {
+        R Jo[9], Jn[9];
+#pragma unroll
+        for (int k = 0; k < 9; k++) {
+            const R* Jk = J + k * L.N;
+            R f[8];
+#pragma unroll
+            for (int c = 0; c < 8; c++) f[c] = Jk[ix[c]];
+            Jo[k] = W.wide_sum(f);
+            Jn[k] = to_real<R>(Jnew[k * L.N + v]);
+        }
+        dphi_of<R, R>(Jn, Jo, Dp);
+    }
+    R sgn;
+    if (!metric_node<R, double>(g6, dg18, L.N, v, geo_new, L.N, v, sgn)) {
+        atomicOr(bad, 1);
+        sgn = geo_new[v];
+    }
     R in[20];
 #pragma unroll
     for (int k = 0; k < 20; k++) {
+        const R* m = mf + k * L.N;
         R s = R(0);
 #pragma unroll
-        for (int c = 0; c < 8; c++) s += R(w[c]) * mf[k * L.N + ix[c]];
+        for (int c = 0; c < 8; c++) s += W.weight(c) * m[ix[c]];
         in[k] = s;
     }
     const R j[3] = {in[1], in[2], in[3]}, B[3] = {in[11], in[12], in[13]};
     const R M2[6] = {in[4], in[5], in[6], in[7], in[8], in[9]};
     const R Cs[6] = {in[14], in[15], in[16], in[17], in[18], in[19]};
-    transform_store<S, R>(L, Pout, hout, geo_new[v], x, y, z, v, Dp, in[0], j, M2, in[10], B, Cs, literal);
+    transform_store<S, R>(L, Pout, hout, sgn, x, y, z, v, Dp, in[0], j, M2, in[10], B, Cs, literal);
 }
 
 // ---------------------------------------------------------------------------
@@ -957,14 +1041,15 @@ template <class S, class R> struct Launch {
                                                                       G(c, 1 - c->gc), (R*)c->J, g6, dg18, Jnew,
                                                                       c->p.transform_flags & 1, bad);
     }
-    static void transform_interp(const cslbm_ctx* c, const double* Jnew, const double* psi3, void* scratch)
+    static void transform_interp(const cslbm_ctx* c, const double* g6, const double* dg18, const double* Jnew,
+                                 const double* psi3, void* scratch, int* bad)
     {
         const int lit = c->p.transform_flags & 1;
         k_moment_fields<S, R><<<nblocks(c->N), TPB, 0, c->stream>>>(make_lat(c), P(c, c->pc), H(c, c->hc), G(c, c->gc),
                                                                    (R*)scratch, lit);
-        k_transform_interp<S, R><<<nblocks(c->N), TPB, 0, c->stream>>>(make_lat(c), P(c, 1 - c->pc), H(c, 1 - c->hc),
-                                                                      G(c, 1 - c->gc), (R*)c->J, Jnew, psi3,
-                                                                      (const R*)scratch, lit);
+        k_transform_interp<S, R><<<(unsigned)((c->N + 127) / 128), 128, 0, c->stream>>>(
+            make_lat(c), P(c, 1 - c->pc), H(c, 1 - c->hc), G(c, 1 - c->gc), (const R*)c->J, g6, dg18, Jnew, psi3,
+            (const R*)scratch, lit, bad);
     }
     static void readout(const cslbm_ctx* c, double* rho, double* u3, long long stride, long long v0, long long cnt,
                         int cartesian)
