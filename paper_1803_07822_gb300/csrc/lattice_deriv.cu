@@ -10,10 +10,16 @@
 // continued by the polynomial of degree `order` through the order + 1 nodes
 // nearest the face, axis by axis (tensor product at edges and corners).
 //
-// Two kernels: k_pad writes F = f - (c_s^2/2) L f (order 4) or the continued f
-// (order 2) on the lattice padded by one site along every axis with a
-// non-periodic face, k_grad forms G_i F at every node from the nine opposite
-// pairs.  One thread per (padded site or node, component); FP64 throughout.
+// Two kernels: the first writes F / 12, F = f - (c_s^2/2) L f (order 4,
+// k_correct) or the continued f (order 2, k_pad), on the lattice padded by one
+// site along every axis with a non-periodic face; k_grad forms G_i F at every
+// node.  FP64 throughout, which is what bounds both: the FP64 pipe issues two
+// lanes per clock and SM, so only the number of FP64 instructions counts.
+// Written out per node, the stencils take 22 and 24 of them; both factor into
+// sums along one axis that neighbours share, which leaves 10 and 15: blocks
+// march along axis 2 with one plane of a 32 x 8 tile (and its rim) in shared
+// memory, in-plane sums exchanged there, sums along the march kept in
+// registers.  Six fields on 128 x 256 x 128, order 4: 1,359 + 1,150 -> 695 + 840 us.
 #include <cstdint>
 #include <string>
 
@@ -26,7 +32,6 @@ namespace cslbm {
 namespace lder {
 
 constexpr int TBL = 256;
-constexpr double kCs2 = 1.0 / 3.0;
 
 struct Box {
     int n[3];
@@ -104,117 +109,209 @@ __device__ __forceinline__ bool inner(const Box& B, int a, int r)
 {
     return r >= 0 && r < B.n[a] && (r >= 1 || B.plo[a]) && (r <= B.n[a] - 2 || B.phi[a]);
 }
-__device__ __forceinline__ long long nb_index(const Box& B, int x, int y, int z)
-{
-    wrap(B, 0, x);
-    wrap(B, 1, y);
-    wrap(B, 2, z);
-    return ((long long)z * B.n[1] + y) * B.n[0] + x;
-}
+// The fields and the weights.  The faces of G_i weigh w_1 / c_s^2 = 1/6, its
+// edges w_7 / c_s^2 = 1/12; the scratch holds F / 12, so that the gradient
+// below needs no products but by two.
+constexpr double kEdge = 1.0 / 12.0;
 
-// F = f - (c_s^2/2) L f = f0 - sum_l w_l (f_l - f0) (order 4), or the
-// continued f (order 2), at every site of the padded lattice; component
-// blockIdx.y
-__global__ void __launch_bounds__(TBL) k_pad(const __grid_constant__ Box B, const double* __restrict__ f, int order,
+// order 2: the continued field at every site of the padded lattice, component blockIdx.y
+__global__ void __launch_bounds__(TBL) k_pad(const __grid_constant__ Box B, const double* __restrict__ f,
                                              double* __restrict__ F)
 {
     // 32-bit site arithmetic (the padded lattice has fewer than 2^32 sites)
     const unsigned s = blockIdx.x * TBL + threadIdx.x;
     if (s >= (unsigned)B.Ne) return;
-    const double* fc = f + (long long)blockIdx.y * B.N;
     const unsigned ne0 = B.ne[0], ne1 = B.ne[1], row = s / ne0, zr = row / ne1;
-    const int x = (int)(s - row * ne0) - B.pad[0];
-    const int y = (int)(row - zr * ne1) - B.pad[1];
-    const int z = (int)zr - B.pad[2];
-    // with sum_{l>0} w_l = 2/3, w = 1/18 on the six faces, 1/36 on the twelve
-    // edges: F = (5/3) f0 - (S_faces + S_edges / 2) / 18
-    double f0, sf = 0.0, se = 0.0;
-    if (inner(B, 0, x) && inner(B, 1, y) && inner(B, 2, z)) {
-        // neighbour offsets per axis, wrapped on periodic axes (as nb_index)
-        const unsigned n0 = B.n[0], n01 = n0 * (unsigned)B.n[1];
-        unsigned o[3][3];
-        const int r[3] = {x, y, z};
-        const unsigned st[3] = {1u, n0, n01};
-#pragma unroll
-        for (int a = 0; a < 3; a++)
-#pragma unroll
-            for (int c = -1; c <= 1; c++) {
-                int q = r[a] + c;
-                wrap(B, a, q);
-                o[a][c + 1] = (unsigned)q * st[a];
-            }
-        f0 = __ldg(fc + (o[2][1] + o[1][1] + o[0][1]));
-        if (order == 4) {
-#pragma unroll
-            for (int l = 1; l < Q; l++) {
-                const double fl = __ldg(fc + (o[2][cvec(l, 2) + 1] + o[1][cvec(l, 1) + 1] + o[0][cvec(l, 0) + 1]));
-                if (l <= 6) sf += fl;
-                else se += fl;
-            }
+    F[(long long)blockIdx.y * B.Ne + s] =
+        kEdge * site(B, f + (long long)blockIdx.y * B.N, 2, (int)(s - row * ne0) - B.pad[0],
+                     (int)(row - zr * ne1) - B.pad[1], (int)zr - B.pad[2]);
+}
+
+// F = f - (c_s^2/2) L f = f0 - sum_l w_l (f_l - f0) at a site whose stencil
+// needs the continuation: with sum_{l>0} w_l = 2/3, w = 1/18 on the six faces,
+// 1/36 on the twelve edges, F = (5/3) f0 - (S_faces + S_edges / 2) / 18
+__device__ __noinline__ double correct_far(const Box& B, const double* __restrict__ f, int x, int y, int z)
+{
+    const double f0 = site(B, f, 4, x, y, z);
+    double sf = 0.0, se = 0.0;
+#pragma unroll 1
+    for (int l = 1; l < Q; l++) {
+        // l = 1..6 faces, 7..18 the edges in the order xy, xz, yz
+        int c[3] = {0, 0, 0};
+        if (l <= 6) {
+            c[(l - 1) >> 1] = l & 1 ? 1 : -1;
+        } else {
+            const int e = (l - 7) >> 2, m = (l - 7) & 3;
+            c[e == 2 ? 1 : 0] = m & 1 ? -1 : 1;
+            c[e == 0 ? 1 : 2] = m & 2 ? -1 : 1;
         }
-    } else {
-        f0 = site(B, fc, order, x, y, z);
-        if (order == 4) {
-#pragma unroll
-            for (int l = 1; l < Q; l++) {
-                const double fl = site(B, fc, order, x + cvec(l, 0), y + cvec(l, 1), z + cvec(l, 2));
-                if (l <= 6) sf += fl;
-                else se += fl;
-            }
-        }
+        const double fl = site(B, f, 4, x + c[0], y + c[1], z + c[2]);
+        if (l <= 6) sf += fl;
+        else se += fl;
     }
-    const double out = order == 4 ? fma(5.0 / 3.0, f0, -fma(0.5, se, sf) * (1.0 / 18.0)) : f0;
-    F[(long long)blockIdx.y * B.Ne + s] = out;
+    return fma(5.0 / 3.0, f0, -fma(0.5, se, sf) * (1.0 / 18.0));
 }
 
-// a site at most one step beyond a face, in the padded lattice
-__device__ __forceinline__ long long pad_index(const Box& B, int x, int y, int z)
+// Tiles of the marching kernels: TX x TY columns, one thread each, by a chunk
+// of planes; the block index counts tiles along axis 0, then 1, then chunks.
+constexpr int TX = 32, TY = 8;
+struct Tiles {
+    int nx, ny, chunk, first, last;  // planes first .. last - 1 in chunks of `chunk`
+};
+__device__ __forceinline__ void tile_of(const Tiles& T, int lo0, int lo1, int& x0, int& y0, int& za, int& zb)
 {
-    wrap(B, 0, x);
-    wrap(B, 1, y);
-    wrap(B, 2, z);
-    return ((long long)(z + B.pad[2]) * B.ne[1] + (y + B.pad[1])) * B.ne[0] + (x + B.pad[0]);
+    const int b = blockIdx.x, bx = b % T.nx, r = b / T.nx, by = r % T.ny, bz = r / T.ny;
+    x0 = lo0 + bx * TX;
+    y0 = lo1 + by * TY;
+    za = T.first + bz * T.chunk;
+    zb = min(T.last, za + T.chunk);
 }
 
-// d_k f_c = G_k F at every node, over the nine opposite pairs:
-// out[(k ncomp + c) N + v]
-__global__ void __launch_bounds__(TBL) k_grad(const __grid_constant__ Box B, int ncomp, const double* __restrict__ F,
-                                              double* __restrict__ out)
+// Order 4: F / 12 on the padded lattice.  With the in-plane sums q = s_x + s_y
+// (s_a = f(a + 1) + f(a - 1)) and e = s_x(y + 1) + s_x(y - 1), and u = f + q/2,
+//   F = (5/3) f - (q + e/2) / 18 - (u(z + 1) + u(z - 1)) / 18.
+// Planes beyond a face of axis 2 continue u and the in-plane part; a site whose
+// stencil leaves the lattice across axis 0 or 1 takes correct_far.
+__global__ void __launch_bounds__(TX* TY) k_correct(const __grid_constant__ Box B, const __grid_constant__ Tiles T,
+                                                    const double* __restrict__ f, double* __restrict__ F)
 {
-    const unsigned v = blockIdx.x * TBL + threadIdx.x;
-    if (v >= (unsigned)B.N) return;
+    __shared__ double fs[TY + 2][TX + 2], ss[TY + 2][TX];
+    const int tx = threadIdx.x, ty = threadIdx.y, t = ty * TX + tx;
+    int x0, y0, za, zb;
+    tile_of(T, -B.pad[0], -B.pad[1], x0, y0, za, zb);
+    const int x = x0 + tx, y = y0 + ty;
+    const double* fc = f + (long long)blockIdx.y * B.N;
+    double* Fc = F + (long long)blockIdx.y * B.Ne;
+    const bool mine = x < B.n[0] + B.pad[0] && y < B.n[1] + B.pad[1];
+    const bool flat = mine && inner(B, 0, x) && inner(B, 1, y);
+    // the tile's entries this thread loads: in-plane offset, or -1 for none
+    int off[2];
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+        const int i = t + k * TX * TY, ly = i / (TX + 2), lx = i - ly * (TX + 2);
+        int rx = x0 - 1 + lx, ry = y0 - 1 + ly;
+        off[k] = -1;
+        if (i < (TX + 2) * (TY + 2) && rx <= B.n[0] && ry <= B.n[1] && wrap(B, 0, rx) && wrap(B, 1, ry))
+            off[k] = ry * B.n[0] + rx;
+    }
+    const unsigned n01 = (unsigned)B.n[0] * B.n[1];
+    // u and the in-plane part w of F at plane pz of the lattice (every thread of the block)
+    auto plane = [&](int pz, double& u, double& w) {
+        const double* fp = fc + (unsigned)pz * n01;
+#pragma unroll
+        for (int k = 0; k < 2; k++)
+            if (off[k] >= 0) (&fs[0][0])[t + k * TX * TY] = __ldg(fp + off[k]);
+        __syncthreads();
+        const double sx = fs[ty + 1][tx] + fs[ty + 1][tx + 2];
+        ss[ty + 1][tx] = sx;
+        if (ty < 2) ss[ty * (TY + 1)][tx] = fs[ty * (TY + 1)][tx] + fs[ty * (TY + 1)][tx + 2];
+        const double f0 = fs[ty + 1][tx + 1], q = sx + (fs[ty][tx + 1] + fs[ty + 2][tx + 1]);
+        __syncthreads();
+        const double e = ss[ty][tx] + ss[ty + 2][tx];
+        u = fma(0.5, q, f0);
+        w = fma(5.0 / 3.0 * kEdge, f0, (-kEdge / 18.0) * fma(0.5, e, q));
+    };
+    double ua = 0.0, ub = 0.0, wb = 0.0;  // u of planes p - 2 and p - 1, w of p - 1
+    for (int p = za - 1; p <= zb; p++) {
+        double u = 0.0, w = 0.0;
+        int pz = p;
+        if (wrap(B, 2, pz)) {
+            plane(pz, u, w);
+        } else {
+            // one or two planes beyond a face: u and w are linear in f, so they
+            // continue with the weights of f
+            const int beyond = p < 0 ? -p : p - (B.n[2] - 1);
+#pragma unroll 1
+            for (int k = 0; k <= 4; k++) {
+                double uk, wk;
+                plane(p < 0 ? k : B.n[2] - 1 - k, uk, wk);
+                const double a = cont_weight(4, beyond, k);
+                u = fma(a, uk, u);
+                w = fma(a, wk, w);
+            }
+        }
+        const int z = p - 1;
+        if (p > za && mine) {
+            const double v = flat ? fma(-kEdge / 18.0, ua + u, wb) : kEdge * correct_far(B, fc, x, y, z);
+            Fc[((unsigned)(z + B.pad[2]) * B.ne[1] + (unsigned)(y + B.pad[1])) * (unsigned)B.ne[0] +
+               (unsigned)(x + B.pad[0])] = v;
+        }
+        ua = ub;
+        ub = u;
+        wb = w;
+    }
+}
+
+// d_k f_c = G_k F at every node, out[(k ncomp + c) N + v].  With the
+// differences d_x = F(x + 1) - F(x - 1), d_y, their sums over the two
+// neighbours across (along y or x in the plane, along z in the march) and
+// z = 2 F + s_x + s_y, in units of F / 12:
+//   D_x = 2 d_x + (d_x(y + 1) + d_x(y - 1)) + (d_x(z + 1) + d_x(z - 1)),
+//   D_y likewise, D_z = z(z + 1) - z(z - 1).
+__global__ void __launch_bounds__(TX* TY) k_grad(const __grid_constant__ Box B, const __grid_constant__ Tiles T, int ncomp,
+                                                 const double* __restrict__ F, double* __restrict__ out)
+{
+    __shared__ double fs[TY + 2][TX + 2], dxs[TY + 2][TX], dys[TY][TX + 2];
+    const int tx = threadIdx.x, ty = threadIdx.y, t = ty * TX + tx;
+    int x0, y0, za, zb;
+    tile_of(T, 0, 0, x0, y0, za, zb);
+    const int x = x0 + tx, y = y0 + ty;
     const int c = blockIdx.y;
     const double* Fc = F + (long long)c * B.Ne;
-    const unsigned n0 = B.n[0], n1 = B.n[1], row = v / n0, zr = row / n1;
-    const int x = (int)(v - row * n0), y = (int)(row - zr * n1), z = (int)zr;
-    // offsets of the sites r + c per axis in the padded lattice (as pad_index)
-    unsigned o[3][3];
-    {
-        const int r[3] = {x, y, z};
-        const unsigned st[3] = {1u, (unsigned)B.ne[0], (unsigned)B.ne[0] * (unsigned)B.ne[1]};
+    const bool mine = x < B.n[0] && y < B.n[1];
+    int off[2];
 #pragma unroll
-        for (int a = 0; a < 3; a++)
-#pragma unroll
-            for (int cc = -1; cc <= 1; cc++) {
-                int q = r[a] + cc;
-                wrap(B, a, q);
-                o[a][cc + 1] = (unsigned)(q + B.pad[a]) * st[a];
-            }
+    for (int k = 0; k < 2; k++) {
+        const int i = t + k * TX * TY, ly = i / (TX + 2), lx = i - ly * (TX + 2);
+        int rx = x0 - 1 + lx, ry = y0 - 1 + ly;
+        off[k] = -1;
+        if (i < (TX + 2) * (TY + 2) && rx <= B.n[0] && ry <= B.n[1]) {
+            wrap(B, 0, rx);
+            wrap(B, 1, ry);
+            off[k] = (ry + B.pad[1]) * B.ne[0] + (rx + B.pad[0]);
+        }
     }
-    double g0 = 0.0, g1 = 0.0, g2 = 0.0;
+    const unsigned ne01 = (unsigned)B.ne[0] * B.ne[1];
+    double dxa = 0.0, dxb = 0.0, rxb = 0.0, dya = 0.0, dyb = 0.0, ryb = 0.0, qa = 0.0, qb = 0.0;
+    for (int p = za - 1; p <= zb; p++) {
+        int pz = p;
+        wrap(B, 2, pz);
+        const double* fp = Fc + (unsigned)(pz + B.pad[2]) * ne01;
 #pragma unroll
-    for (int k = 0; k < 9; k++) {
-        const int l = 2 * k + 1, cx = cvec(l, 0), cy = cvec(l, 1), cz = cvec(l, 2);
-        const double d = __ldg(Fc + (o[2][cz + 1] + o[1][cy + 1] + o[0][cx + 1])) -
-                         __ldg(Fc + (o[2][1 - cz] + o[1][1 - cy] + o[0][1 - cx]));
-        const double wd = wq(l) / kCs2;
-        if (cx) g0 = fma(cx * wd, d, g0);
-        if (cy) g1 = fma(cy * wd, d, g1);
-        if (cz) g2 = fma(cz * wd, d, g2);
+        for (int k = 0; k < 2; k++)
+            if (off[k] >= 0) (&fs[0][0])[t + k * TX * TY] = __ldg(fp + off[k]);
+        __syncthreads();
+        const double e = fs[ty + 1][tx + 2], w = fs[ty + 1][tx], n = fs[ty + 2][tx + 1], s = fs[ty][tx + 1];
+        const double dx = e - w, dy = n - s;
+        dxs[ty + 1][tx] = dx;
+        dys[ty][tx + 1] = dy;
+        // the rims: d_x of the rows beside the tile, d_y of the columns
+        if (ty < 2) dxs[ty * (TY + 1)][tx] = fs[ty * (TY + 1)][tx + 2] - fs[ty * (TY + 1)][tx];
+        else if (ty == 2 && tx < 2 * TY) {
+            const int r = tx >> 1, col = (tx & 1) * (TX + 1);
+            dys[r][col] = fs[r + 2][col] - fs[r][col];
+        }
+        const double q = fma(2.0, fs[ty + 1][tx + 1], (e + w) + (n + s));
+        __syncthreads();
+        const double rx = fma(2.0, dx, dxs[ty][tx] + dxs[ty + 2][tx]);
+        const double ry = fma(2.0, dy, dys[ty][tx] + dys[ty][tx + 2]);
+        if (p > za && mine) {
+            const unsigned v = ((unsigned)(p - 1) * B.n[1] + (unsigned)y) * (unsigned)B.n[0] + (unsigned)x;
+            double* o = out + (long long)c * B.N + v;
+            const long long comp = (long long)ncomp * B.N;
+            o[0] = rxb + (dxa + dx);
+            o[comp] = ryb + (dya + dy);
+            o[2 * comp] = q - qa;
+        }
+        dxa = dxb;
+        dxb = dx;
+        rxb = rx;
+        dya = dyb;
+        dyb = dy;
+        ryb = ry;
+        qa = qb;
+        qb = q;
     }
-    out[((long long)0 * ncomp + c) * B.N + v] = g0;
-    out[((long long)1 * ncomp + c) * B.N + v] = g1;
-    out[((long long)2 * ncomp + c) * B.N + v] = g2;
 }
 
 Box box_of(const cslbm_ctx* c, int order)
@@ -256,6 +353,25 @@ bool device_memory(const void* p)
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// Chunks of at most 32 planes (a march repeats two planes of its neighbours'),
+// shorter ones while there are fewer than eight blocks per SM
+Tiles tiles_of(const cslbm_ctx* c, int e0, int e1, int first, int last, int ncomp)
+{
+    Tiles T;
+    T.nx = (e0 + TX - 1) / TX;
+    T.ny = (e1 + TY - 1) / TY;
+    T.first = first;
+    T.last = last;
+    T.chunk = 32;
+    while (T.chunk > 4 && (long long)T.nx * T.ny * ncomp * ((last - first + T.chunk - 1) / T.chunk) < 8LL * c->n_sm)
+        T.chunk /= 2;
+    return T;
+}
+dim3 tile_grid(const Tiles& T, int ncomp)
+{
+    return dim3((unsigned)T.nx * T.ny * ((T.last - T.first + T.chunk - 1) / T.chunk), (unsigned)ncomp);
+}
+
 size_t pad_bytes(const cslbm_ctx* c, int ncomp, int order)
 {
     return (size_t)ncomp * (size_t)box_of(c, order).Ne * sizeof(double);
@@ -271,8 +387,14 @@ cslbm_status gradient(cslbm_ctx* c, const double* f, int ncomp, int order, doubl
         return lfail(CSLBM_EINVAL, "fields, output and scratch must be device memory");
     const Box B = box_of(c, order);
     double* F = (double*)scratch;
-    k_pad<<<dim3((unsigned)((B.Ne + TBL - 1) / TBL), (unsigned)ncomp), TBL, 0, c->stream>>>(B, f, order, F);
-    k_grad<<<dim3((unsigned)((B.N + TBL - 1) / TBL), (unsigned)ncomp), TBL, 0, c->stream>>>(B, ncomp, F, out);
+    if (order == 4) {
+        const Tiles T = tiles_of(c, B.ne[0], B.ne[1], -B.pad[2], B.n[2] + B.pad[2], ncomp);
+        k_correct<<<tile_grid(T, ncomp), dim3(TX, TY), 0, c->stream>>>(B, T, f, F);
+    } else {
+        k_pad<<<dim3((unsigned)((B.Ne + TBL - 1) / TBL), (unsigned)ncomp), TBL, 0, c->stream>>>(B, f, F);
+    }
+    const Tiles T = tiles_of(c, B.n[0], B.n[1], 0, B.n[2], ncomp);
+    k_grad<<<tile_grid(T, ncomp), dim3(TX, TY), 0, c->stream>>>(B, T, ncomp, F, out);
     c->launches += 2;
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return lfail(CSLBM_ECUDA, std::string("lattice gradient: ") + cudaGetErrorString(e));
