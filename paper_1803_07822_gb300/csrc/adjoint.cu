@@ -4,26 +4,35 @@
 // One backward step takes the adjoint of the state at time t+1 (populations
 // and history, "lambda") to time t, given the forward state at time t in the
 // context, and adds the step's contribution to the adjoint of the geometry.
-// The step's dependencies are local except three, each handled by a pass of
-// its own:
+// The adjoint of the populations is kept per node that pulls them (field lS:
+// the adjoint of stored slot (l, y) is lS_l of node y + c_l, zero where that
+// is a face node, whose pulled values the boundary rule ignores), so that the
+// pull reversed is the gather of the next pass A and no pass of its own.
+// The step's dependencies are local except three:
 //   A  (every node) the forward step of the node recomputed and reversed
-//      (adj::step_reverse): adjoints of its pulled populations (field lS),
-//      of its history at t (lH at t), of its geometry (lGeo, accumulated)
-//      and of its lattice gradient D (field lD).  A face node reverses the
-//      ghost extrapolation of its stencil and adds the rho-u adjoint of the
-//      real sites to lJF with atomics;
+//      (adj::step_reverse) from lS gathered at y + c_l: adjoints of its pulled
+//      populations (the other lS buffer), of its history at t (lH at t), of
+//      its geometry (lGeo, accumulated) and of its lattice gradient D (field
+//      lD).  A face node reverses the ghost extrapolation of its stencil and
+//      adds the rho-u adjoint of the real sites to lJF with atomics;
 //   B  (every node y) the rho-u adjoint of y gathered from the lD of the
 //      interior nodes whose stencil holds y, plus lJF; since
 //      j(y) = sqrt(g) sum_l s_l c_l + B(y)/2 it goes to lS(y), to sqrt(g)
 //      and to the history B of y;
 //   C  (face nodes) the boundary rule reversed: lS of the face node goes to
 //      the pulled populations of its inner node, both nodes' metric and
-//      history (atomics: edge and corner nodes share inner nodes);
-//   D  (every slot) the pull reversed: the adjoint of stored value (l, y) is
-//      lS_l of the node that pulls it, y + c_l, or zero when that node is a
-//      face node (the boundary rule ignores its pulled values).
+//      history (atomics: edge and corner nodes share inner nodes); lS of the
+//      face node becomes zero.
 // A pass's forward quantities come from the context's state at time t and
 // from rho u at time t, which the backward step recomputes first.
+//
+// Pass A is bound by the latency of its loads (about 700 B per node at 128
+// registers), so the 89 values of a node that the arithmetic needs late --
+// geometry, histories, the gathered lS, the geometry adjoint -- travel to
+// shared memory asynchronously and face nodes run in blocks of their own; B
+// reads the 90 lD values of a node's neighbours without a face test (lD of a
+// face node is zero).  64 x 128 x 64 FP32, us per backward step: A 175 -> 112,
+// the pull of a pass of its own 29 -> 0.
 #include <cstdio>
 #include <string>
 
@@ -34,12 +43,9 @@
 namespace cslbm {
 namespace adj {
 
-constexpr int TB_A = 128;
-
 template <class R> struct Bufs {
-    R* lP[2];   // [19][N] adjoint of the stored populations (current: lp)
+    R* lS[2];   // [19][N] adjoint of each node's pulled (face node: rule) populations (current: lp)
     R* lH[2];   // [10][N] adjoint of the history
-    R* lS;      // [19][N] adjoint of each node's pulled (face node: rule) populations
     R* lD;      // [9][N]  adjoint of each node's lattice gradient D[k][i] at k*3+i
     R* lJF;     // [3][N]  rho-u adjoint scattered by face nodes
     R* lGeo;    // [25][N] adjoint of the geometry, summed over the steps
@@ -47,15 +53,6 @@ template <class R> struct Bufs {
 };
 
 template <class R> __device__ __forceinline__ void add(R* p, R v) { atomicAdd(p, v); }
-
-// (32-bit arithmetic: a context holds fewer than 2^32 nodes)
-__device__ __forceinline__ void node_xyz(const Lat& L, long long v, int& x, int& y, int& z)
-{
-    const unsigned vu = (unsigned)v, n0 = L.n[0], n1 = L.n[1], row = vu / n0, zr = row / n1;
-    x = (int)(vu - row * n0);
-    y = (int)(row - zr * n1);
-    z = (int)zr;
-}
 
 // ghost extrapolation of a stencil site reversed: the adjoint lj of the
 // site's rho u distributed onto the real nodes it was built from
@@ -97,63 +94,27 @@ __device__ __noinline__ void face_inputs(const Lat& L, const R* __restrict__ P, 
     }
 }
 
-// pass A
+// pass A: threads per block (the staged values of a block fit the static 48 KB)
+template <class R> constexpr int kTA = sizeof(R) == 8 ? 64 : 128;
+// staged values of a node: geometry, history, adjoint of the new history,
+// gathered adjoint of the new populations, geometry adjoint
+constexpr int S_H = NGEO, S_LH = S_H + NHIST, S_LP = S_LH + NHIST, S_LG = S_LP + Q, S_ALL = S_LG + NG;
+
+// the part of pass A that face and interior nodes share: from the forward
+// inputs and the adjoints of the outputs to the stored adjoints; lD returned
 template <class R>
-__global__ void __launch_bounds__(TB_A, 4) k_adj_local(Lat L, const R* __restrict__ P, const R* __restrict__ H,
-                                                     const R* __restrict__ geo, const Mom4<R>* __restrict__ jf,
-                                                     const R* __restrict__ lPo, const R* __restrict__ lHo,
-                                                     Bufs<R> B, R* __restrict__ lHi)
+__device__ __forceinline__ void local_reverse(const Lat& L, const R (&s)[Q], const GeoT<R>& G, const HistT<R>& Hp,
+                                              const R (&d)[9][3], const R (&lout)[Q], const HistT<R>& lH,
+                                              R* __restrict__ lSn, R* __restrict__ lHi, R (&lgeo)[NG], R (&lD)[3][3],
+                                              unsigned v, size_t N)
 {
-    // 32-bit node arithmetic (a context holds fewer than 2^32 nodes)
-    const unsigned vu = blockIdx.x * TB_A + threadIdx.x;
-    if (vu >= (unsigned)L.N) return;
-    const long long v = vu, N = L.N;
-    const unsigned n0 = L.n[0], n1 = L.n[1], row = vu / n0, zr = row / n1;
-    const int x = (int)(vu - row * n0), y = (int)(row - zr * n1), z = (int)zr;
-    const bool face = on_boundary(L, x, y, z);
-    R s[Q];
-    R d[9][3];
-    if (face) {
-        R sf[Q], df[27];
-        face_inputs<R>(L, P, H, geo, jf, x, y, z, sf, df);
-#pragma unroll
-        for (int l = 0; l < Q; l++) s[l] = sf[l];
-#pragma unroll
-        for (int k = 0; k < 9; k++)
-#pragma unroll
-            for (int i = 0; i < 3; i++) d[k][i] = df[3 * k + i];
-    } else {
-        gather_raw<R, R>(L, P, x, y, z, s);
-        const Nbr nb = nbr_index(L, x, y, z, +1);  // sites x + c, wrapped
-#pragma unroll
-        for (int k = 0; k < 9; k++) {
-            const int l = 2 * k + 1, cx = cvec(l, 0), cy = cvec(l, 1), cz = cvec(l, 2);
-            const Mom4<R> p = jf[nbr_off(nb, cx, cy, cz)], m = jf[nbr_off(nb, -cx, -cy, -cz)];
-            d[k][0] = p.x - m.x;
-            d[k][1] = p.y - m.y;
-            d[k][2] = p.z - m.z;
-        }
-    }
-    GeoT<R> G;
-    HistT<R> Hp;
-    load_geo_hist(geo, H, (unsigned)v, (unsigned)N, G, Hp);
-    R lout[Q];
-#pragma unroll
-    for (int l = 0; l < Q; l++) lout[l] = lPo[l * N + v];
-    HistT<R> lH, lHp;
-    lH.A = lHo[v];
+    HistT<R> lHp;
     lHp.A = R(0);
 #pragma unroll
-    for (int a = 0; a < 3; a++) {
-        lH.B[a] = lHo[(1 + a) * N + v];
-        lHp.B[a] = R(0);
-    }
+    for (int a = 0; a < 3; a++) lHp.B[a] = R(0);
 #pragma unroll
-    for (int k = 0; k < 6; k++) {
-        lH.C[k] = lHo[(4 + k) * N + v];
-        lHp.C[k] = R(0);
-    }
-    R ls[Q], lgeo[NG], lD[3][3];
+    for (int k = 0; k < 6; k++) lHp.C[k] = R(0);
+    R ls[Q];
 #pragma unroll
     for (int l = 0; l < Q; l++) ls[l] = R(0);
 #pragma unroll
@@ -164,49 +125,52 @@ __global__ void __launch_bounds__(TB_A, 4) k_adj_local(Lat L, const R* __restric
         for (int i = 0; i < 3; i++) lD[k][i] = R(0);
     step_reverse(L, s, G, Hp, d, lout, lH, ls, lHp, lgeo, lD);
 #pragma unroll
-    for (int l = 0; l < Q; l++) B.lS[l * N + v] = ls[l];
+    for (int l = 0; l < Q; l++) lSn[l * N + v] = ls[l];
     lHi[v] = lHp.A;
 #pragma unroll
     for (int a = 0; a < 3; a++) lHi[(1 + a) * N + v] = lHp.B[a];
 #pragma unroll
     for (int k = 0; k < 6; k++) lHi[(4 + k) * N + v] = lHp.C[k];
-#pragma unroll
-    for (int k = 0; k < NG; k++) B.lGeo[k * N + v] += lgeo[k];
-    if (face) {
-        R ld[9][3];
-        gradient_reverse(lD, ld);
-#pragma unroll
-        for (int k = 0; k < 9; k++) {
-            const int l = 2 * k + 1, cx = cvec(l, 0), cy = cvec(l, 1), cz = cvec(l, 2);
-            site_reverse(L, x + cx, y + cy, z + cz, ld[k][0], ld[k][1], ld[k][2], B.lJF);
-            site_reverse(L, x - cx, y - cy, z - cz, -ld[k][0], -ld[k][1], -ld[k][2], B.lJF);
-        }
-#pragma unroll
-        for (int q = 0; q < 9; q++) B.lD[q * N + v] = R(0);
-    } else {
-#pragma unroll
-        for (int k = 0; k < 3; k++)
-#pragma unroll
-            for (int i = 0; i < 3; i++) B.lD[(k * 3 + i) * N + v] = lD[k][i];
-    }
 }
 
-// pass B
 template <class R>
-__global__ void __launch_bounds__(256) k_adj_gather(Lat L, const R* __restrict__ H, const R* __restrict__ geo,
-                                                     const Mom4<R>* __restrict__ jf, Bufs<R> B, R* __restrict__ lHi)
+__device__ __forceinline__ void load_lhist(const R* __restrict__ lHo, unsigned v, size_t N, HistT<R>& lH)
 {
-    const long long v = blockIdx.x * 256LL + threadIdx.x;
-    if (v >= L.N) return;
-    const long long N = L.N;
-    int x, y, z;
-    node_xyz(L, v, x, y, z);
-    R lj[3] = {B.lJF[v], B.lJF[N + v], B.lJF[2 * N + v]};
-    // interior nodes x' = y - c whose stencil site x' + c is this node
+    lH.A = lHo[v];
 #pragma unroll
-    for (int l = 1; l < Q; l++) {
-        const int cx = cvec(l, 0), cy = cvec(l, 1), cz = cvec(l, 2);
-        int r[3] = {x - cx, y - cy, z - cz};
+    for (int a = 0; a < 3; a++) lH.B[a] = lHo[(1 + a) * N + v];
+#pragma unroll
+    for (int k = 0; k < 6; k++) lH.C[k] = lHo[(4 + k) * N + v];
+}
+
+template <class R>
+__device__ __noinline__ void local_face(const Lat& L, const R* __restrict__ P, const R* __restrict__ H,
+                                        const R* __restrict__ geo, const Mom4<R>* __restrict__ jf,
+                                        const R* __restrict__ lSo, const R* __restrict__ lHo, R* __restrict__ lSn,
+                                        R* __restrict__ lHi, const Bufs<R>& B, int x, int y, int z)
+{
+    const size_t N = L.N;
+    const unsigned v = (unsigned)nidx(L, x, y, z);
+    R s[Q], d[9][3];
+    {
+        R sf[Q], df[27];
+        face_inputs<R>(L, P, H, geo, jf, x, y, z, sf, df);
+#pragma unroll
+        for (int l = 0; l < Q; l++) s[l] = sf[l];
+#pragma unroll
+        for (int k = 0; k < 9; k++)
+#pragma unroll
+            for (int i = 0; i < 3; i++) d[k][i] = df[3 * k + i];
+    }
+    GeoT<R> G;
+    HistT<R> Hp, lH;
+    load_geo_hist(geo, H, v, (unsigned)N, G, Hp);
+    load_lhist(lHo, v, N, lH);
+    // lS of the nodes that pull from this one (zero at face nodes)
+    R lout[Q];
+#pragma unroll
+    for (int l = 0; l < Q; l++) {
+        int r[3] = {x + cvec(l, 0), y + cvec(l, 1), z + cvec(l, 2)};
         bool ok = true;
 #pragma unroll
         for (int a = 0; a < 3; a++)
@@ -214,35 +178,197 @@ __global__ void __launch_bounds__(256) k_adj_gather(Lat L, const R* __restrict__
                 if ((r[a] < 0 ? L.bclo[a] : L.bchi[a]) == BC_PERIODIC) r[a] = wrapc(r[a], L.n[a]);
                 else ok = false;
             }
-        if (!ok || on_boundary(L, r[0], r[1], r[2])) continue;
-        const long long u = nidx(L, r[0], r[1], r[2]);
+        lout[l] = ok ? lSo[l * N + nidx(L, r[0], r[1], r[2])] : R(0);
+    }
+    R lgeo[NG], lD[3][3];
+    local_reverse<R>(L, s, G, Hp, d, lout, lH, lSn, lHi, lgeo, lD, v, N);
+#pragma unroll
+    for (int k = 0; k < NG; k++) B.lGeo[k * N + v] += lgeo[k];
+    R ld[9][3];
+    gradient_reverse(lD, ld);
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        const int l = 2 * k + 1, cx = cvec(l, 0), cy = cvec(l, 1), cz = cvec(l, 2);
+        site_reverse(L, x + cx, y + cy, z + cz, ld[k][0], ld[k][1], ld[k][2], B.lJF);
+        site_reverse(L, x - cx, y - cy, z - cz, -ld[k][0], -ld[k][1], -ld[k][2], B.lJF);
+    }
+#pragma unroll
+    for (int q = 0; q < 9; q++) B.lD[q * N + v] = R(0);
+}
+
+// pass A: the first nfb blocks take the face nodes, the others the nodes of
+// the planes between non-periodic faces of axis 2, v = v0 .. (as k_step_flat)
+template <class R>
+__global__ void __launch_bounds__(kTA<R>, 4)
+    k_adj_local(const __grid_constant__ Lat L, const __grid_constant__ Plane pl, const __grid_constant__ FaceList f,
+                unsigned nfb, unsigned v0, unsigned v1, const R* __restrict__ P, const R* __restrict__ H,
+                const R* __restrict__ geo, const Mom4<R>* __restrict__ jf, const R* __restrict__ lSo,
+                const R* __restrict__ lHo, R* __restrict__ lSn, R* __restrict__ lHi, const __grid_constant__ Bufs<R> B)
+{
+    constexpr int TA = kTA<R>;
+    __shared__ R stage[S_ALL * TA];
+    int x, y, z;
+    if (blockIdx.x < nfb) {
+        if (face_coords(f, (int)(blockIdx.x * TA + threadIdx.x), x, y, z))
+            local_face<R>(L, P, H, geo, jf, lSo, lHo, lSn, lHi, B, x, y, z);
+        return;
+    }
+    const unsigned v = v0 + (blockIdx.x - nfb) * TA + threadIdx.x;
+    flat_coords(L, pl, v, x, y, z);
+    if (v >= v1 || on_boundary(L, x, y, z)) return;
+    const size_t N = L.N;
+    const unsigned Nu = (unsigned)N;
+    R* sm = stage + threadIdx.x;
+    const Nbr src = nbr_index(L, x, y, z, -1);  // sites x - c, wrapped
+#pragma unroll
+    for (int k = 0; k < NGEO; k++) copy_async(sm + k * TA, geo + k * N + v);
+#pragma unroll
+    for (int k = 0; k < NHIST; k++) copy_async(sm + (S_H + k) * TA, H + k * N + v);
+#pragma unroll
+    for (int l = 0; l < Q; l++)  // lS of the node x + c that pulls population l of this one
+        copy_async(sm + (S_LP + l) * TA, lSo + l * N + nbr_off(src, -cvec(l, 0), -cvec(l, 1), -cvec(l, 2)));
+#pragma unroll
+    for (int k = 0; k < NHIST; k++) copy_async(sm + (S_LH + k) * TA, lHo + k * N + v);
+#pragma unroll
+    for (int k = 0; k < NG; k++) copy_async(sm + (S_LG + k) * TA, B.lGeo + k * N + v);
+    R s[Q], d[9][3];
+#pragma unroll
+    for (int l = 0; l < Q; l++)
+        s[l] = __ldg(P + (unsigned)pslot(l) * Nu + nbr_off(src, cvec(l, 0), cvec(l, 1), cvec(l, 2)));
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        const int l = 2 * k + 1, cx = cvec(l, 0), cy = cvec(l, 1), cz = cvec(l, 2);
+        const Mom4<R> p = jf[nbr_off(src, -cx, -cy, -cz)], m = jf[nbr_off(src, cx, cy, cz)];
+        d[k][0] = p.x - m.x;
+        d[k][1] = p.y - m.y;
+        d[k][2] = p.z - m.z;
+    }
+    copies_landed();
+    GeoT<R> G;
+    HistT<R> Hp, lH;
+    G.sg = sm[0];
+    G.isg = recip(G.sg);
+#pragma unroll
+    for (int a = 0; a < 6; a++) G.gi[a] = sm[(1 + a) * TA];
+#pragma unroll
+    for (int a = 0; a < 18; a++) G.gam[a] = sm[(7 + a) * TA];
+#pragma unroll
+    for (int k = 0; k < 3; k++) G.gc[k] = (G.gam[0 * 6 + s6(k, 0)] + G.gam[1 * 6 + s6(k, 1)]) + G.gam[2 * 6 + s6(k, 2)];
+    Hp.A = sm[S_H * TA];
+    lH.A = sm[S_LH * TA];
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        Hp.B[a] = sm[(S_H + 1 + a) * TA];
+        lH.B[a] = sm[(S_LH + 1 + a) * TA];
+    }
+#pragma unroll
+    for (int a = 0; a < 6; a++) {
+        Hp.C[a] = sm[(S_H + 4 + a) * TA];
+        lH.C[a] = sm[(S_LH + 4 + a) * TA];
+    }
+    R lout[Q];
+#pragma unroll
+    for (int l = 0; l < Q; l++) lout[l] = sm[(S_LP + l) * TA];
+    R lgeo[NG], lD[3][3];
+    local_reverse<R>(L, s, G, Hp, d, lout, lH, lSn, lHi, lgeo, lD, v, N);
+#pragma unroll
+    for (int k = 0; k < NG; k++) B.lGeo[k * N + v] = sm[(S_LG + k) * TA] + lgeo[k];
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+#pragma unroll
+        for (int i = 0; i < 3; i++) B.lD[(k * 3 + i) * N + v] = lD[k][i];
+}
+
+// pass B: the rho-u adjoint of a face node gathered (neighbours past a face are none)
+template <class R>
+__device__ __noinline__ Mom4<R> gather_face(const Lat& L, const R* __restrict__ lD, int x, int y, int z)
+{
+    const size_t N = L.N;
+    R lj[3] = {R(0), R(0), R(0)};
+#pragma unroll
+    for (int l = 1; l < Q; l++) {
+        const int c[3] = {cvec(l, 0), cvec(l, 1), cvec(l, 2)};
+        int r[3] = {x - c[0], y - c[1], z - c[2]};
+        bool ok = true;
+#pragma unroll
+        for (int a = 0; a < 3; a++)
+            if (r[a] < 0 || r[a] >= L.n[a]) {
+                if ((r[a] < 0 ? L.bclo[a] : L.bchi[a]) == BC_PERIODIC) r[a] = wrapc(r[a], L.n[a]);
+                else ok = false;
+            }
+        if (!ok) continue;
+        const unsigned u = (unsigned)nidx(L, r[0], r[1], r[2]);
         const R w = R(3.0 * wq(l));
-        const int c[3] = {cx, cy, cz};
 #pragma unroll
         for (int k = 0; k < 3; k++) {
             if (!c[k]) continue;
 #pragma unroll
-            for (int i = 0; i < 3; i++) lj[i] += w * R(c[k]) * B.lD[(k * 3 + i) * N + u];
+            for (int i = 0; i < 3; i++) lj[i] += w * R(c[k]) * lD[(k * 3 + i) * N + u];
         }
     }
+    return Mom4<R>{lj[0], lj[1], lj[2], R(0)};
+}
+
+template <class R>
+__global__ void __launch_bounds__(FB, sizeof(R) == 8 ? 4 : 8)
+    k_adj_gather(const __grid_constant__ Lat L, const __grid_constant__ Plane pl, const R* __restrict__ H,
+                 const R* __restrict__ geo, const Mom4<R>* __restrict__ jf, R* __restrict__ lS,
+                 const __grid_constant__ Bufs<R> B, R* __restrict__ lHi)
+{
+    const unsigned v = blockIdx.x * FB + threadIdx.x;
+    if (v >= (unsigned)L.N) return;
+    const size_t N = L.N;
+    int x, y, z;
+    flat_coords(L, pl, v, x, y, z);
+    R lj[3];
+    if (on_boundary(L, x, y, z)) {
+        const Mom4<R> g = gather_face<R>(L, B.lD, x, y, z);
+        lj[0] = g.x;
+        lj[1] = g.y;
+        lj[2] = g.z;
+    } else {
+        // interior nodes x' = y - c whose stencil site x' + c is this node
+        const Nbr src = nbr_index(L, x, y, z, -1);
+        const R* lD = B.lD;
+        R face[3] = {R(0), R(0), R(0)}, edge[3] = {R(0), R(0), R(0)};
+#pragma unroll
+        for (int l = 1; l < Q; l++) {
+            const int c[3] = {cvec(l, 0), cvec(l, 1), cvec(l, 2)};
+            const unsigned u = nbr_off(src, c[0], c[1], c[2]);
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                if (!c[k]) continue;
+#pragma unroll
+                for (int i = 0; i < 3; i++) {
+                    const R t = lD[(k * 3 + i) * N + u];
+                    if (l <= 6) face[i] += c[k] > 0 ? t : -t;
+                    else edge[i] += c[k] > 0 ? t : -t;
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 3; i++) lj[i] = fmad(R(1.0 / 6.0), face[i], R(1.0 / 12.0) * edge[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 3; i++) lj[i] += B.lJF[i * N + v];
     // j(y) = sqrt(g) m1 + B/2 with m1 = (j - B/2) / sqrt(g)
-    const R sg = geo[v];
+    const R sg = geo[v], isg = recip(sg);
     const Mom4<R> jv = jf[v];
     const R jj[3] = {jv.x, jv.y, jv.z};
     R lsg = R(0);
 #pragma unroll
     for (int a = 0; a < 3; a++) {
         const R Bh = H[(1 + a) * N + v];
-        lsg += (jj[a] - R(0.5) * Bh) / sg * lj[a];
+        lsg += (jj[a] - R(0.5) * Bh) * isg * lj[a];
         lHi[(1 + a) * N + v] += R(0.5) * lj[a];
     }
     B.lGeo[v] += lsg;
 #pragma unroll
-    for (int l = 0; l < Q; l++) {
+    for (int l = 1; l < Q; l++) {
         R t = R(0);
 #pragma unroll
         for (int a = 0; a < 3; a++) t += R(cvec(l, a)) * lj[a];
-        B.lS[l * N + v] += sg * t;
+        lS[l * N + v] += sg * t;
     }
 }
 
@@ -250,7 +376,8 @@ __global__ void __launch_bounds__(256) k_adj_gather(Lat L, const R* __restrict__
 template <class R>
 __global__ void __launch_bounds__(128) k_adj_boundary(const __grid_constant__ Lat L, const __grid_constant__ FaceList f,
                                                        const R* __restrict__ P, const R* __restrict__ H,
-                                                       const R* __restrict__ geo, Bufs<R> B, R* __restrict__ lHi)
+                                                       const R* __restrict__ geo, R* __restrict__ lS, Bufs<R> B,
+                                                       R* __restrict__ lHi)
 {
     const long long t = blockIdx.x * 128LL + threadIdx.x;
     if (t >= f.start[f.nseg]) return;
@@ -294,7 +421,8 @@ __global__ void __launch_bounds__(128) k_adj_boundary(const __grid_constant__ La
     R ls[Q], lsi[Q], lgi_i[7], lgi_w[7];
 #pragma unroll
     for (int l = 0; l < Q; l++) {
-        ls[l] = B.lS[l * N + vw];
+        ls[l] = lS[l * N + vw];
+        lS[l * N + vw] = R(0);
         lsi[l] = R(0);
     }
 #pragma unroll
@@ -307,7 +435,7 @@ __global__ void __launch_bounds__(128) k_adj_boundary(const __grid_constant__ La
     for (int k = 0; k < 6; k++) lHi_.C[k] = lHw_.C[k] = R(0);
     boundary_reverse(L, bc, si, Gi, Gw, Hi, Hw, uw, ls, lsi, lgi_i, lgi_w, lHi_, lHw_);
 #pragma unroll
-    for (int l = 0; l < Q; l++) add(B.lS + l * N + vi, lsi[l]);
+    for (int l = 0; l < Q; l++) add(lS + l * N + vi, lsi[l]);
 #pragma unroll
     for (int k = 0; k < 7; k++) {
         add(B.lGeo + k * N + vi, lgi_i[k]);
@@ -327,30 +455,6 @@ __global__ void __launch_bounds__(128) k_adj_boundary(const __grid_constant__ La
     }
 }
 
-// pass D: the pull reversed
-template <class R>
-__global__ void __launch_bounds__(256) k_adj_pull(Lat L, const R* __restrict__ lS, R* __restrict__ lPi)
-{
-    const long long v = blockIdx.x * 256LL + threadIdx.x;
-    if (v >= L.N) return;
-    int x, y, z;
-    node_xyz(L, v, x, y, z);
-#pragma unroll
-    for (int l = 0; l < Q; l++) {
-        int r[3] = {x + cvec(l, 0), y + cvec(l, 1), z + cvec(l, 2)};
-        bool ok = true;
-#pragma unroll
-        for (int a = 0; a < 3; a++)
-            if (r[a] < 0 || r[a] >= L.n[a]) {
-                if ((r[a] < 0 ? L.bclo[a] : L.bchi[a]) == BC_PERIODIC) r[a] = wrapc(r[a], L.n[a]);
-                else ok = false;
-            }
-        R val = R(0);
-        if (ok && !on_boundary(L, r[0], r[1], r[2])) val = lS[l * L.N + nidx(L, r[0], r[1], r[2])];
-        lPi[l * L.N + v] = val;
-    }
-}
-
 // seed: the adjoint of e . F (F the force of the fluid on face (axis, side),
 // k_wall_force) onto the face nodes' populations (lS, before the boundary
 // rule), history, geometry and chart Jacobian
@@ -358,7 +462,7 @@ template <class R>
 __global__ void __launch_bounds__(128) k_adj_seed_force(Lat L, const R* __restrict__ P, const R* __restrict__ H,
                                                          const R* __restrict__ geo, const R* __restrict__ J,
                                                          int axis, int side, double e0, double e1, double e2,
-                                                         Bufs<R> B, R* __restrict__ lHo)
+                                                         R* __restrict__ lS, Bufs<R> B, R* __restrict__ lHo)
 {
     const int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
     const long long nf = (long long)L.n[a1] * L.n[a2];
@@ -436,7 +540,7 @@ __global__ void __launch_bounds__(128) k_adj_seed_force(Lat L, const R* __restri
     for (int l = 0; l < Q; l++) ls[l] = R(0);
     moments_reverse(lm0, lm1, lm2, ls);
 #pragma unroll
-    for (int l = 0; l < Q; l++) B.lS[l * N + v] += ls[l];
+    for (int l = 0; l < Q; l++) lS[l * N + v] += ls[l];
     B.lGeo[v] += lsgR;
 #pragma unroll
     for (int k = 0; k < 6; k++) B.lGeo[(1 + k) * N + v] += lgi[k];
@@ -447,29 +551,18 @@ __global__ void __launch_bounds__(128) k_adj_seed_force(Lat L, const R* __restri
     for (int k = 0; k < 6; k++) lHo[(4 + k) * N + v] += lC[k];
 }
 
-// the rest initialisation reversed, every node
+// the rest initialisation reversed, every node (lS of a face node is zero)
 template <class R>
-__global__ void __launch_bounds__(256) k_adj_init(Lat L, const R* __restrict__ geo, const R* __restrict__ lP,
-                                                   const R* __restrict__ lH, R* __restrict__ lGeo)
+__global__ void __launch_bounds__(128) k_adj_init(const __grid_constant__ Lat L, const R* __restrict__ geo,
+                                                   const R* __restrict__ lS, const R* __restrict__ lH,
+                                                   R* __restrict__ lGeo)
 {
-    const long long v = blockIdx.x * 256LL + threadIdx.x;
+    const long long v = blockIdx.x * 128LL + threadIdx.x;
     if (v >= L.N) return;
     const long long N = L.N;
-    int x, y, z;
-    node_xyz(L, v, x, y, z);
     R ls0[Q];
 #pragma unroll
-    for (int l = 0; l < Q; l++) {
-        int r[3] = {x - cvec(l, 0), y - cvec(l, 1), z - cvec(l, 2)};
-        bool ok = true;
-#pragma unroll
-        for (int a = 0; a < 3; a++)
-            if (r[a] < 0 || r[a] >= L.n[a]) {
-                if ((r[a] < 0 ? L.bclo[a] : L.bchi[a]) == BC_PERIODIC) r[a] = wrapc(r[a], L.n[a]);
-                else ok = false;
-            }
-        ls0[l] = ok ? lP[l * N + nidx(L, r[0], r[1], r[2])] : R(0);
-    }
+    for (int l = 0; l < Q; l++) ls0[l] = lS[l * N + v];
     GeoT<R> G;
     HistT<R> dummy;
     load_geo_hist(geo, lH, (unsigned)v, (unsigned)N, G, dummy);
@@ -519,9 +612,8 @@ template <class R> Bufs<R> bufs(const cslbm_ctx* c)
         o += (n + 63) / 64 * 64;
         return q;
     };
-    for (int k = 0; k < 2; k++) B.lP[k] = (R*)take(19 * N * sizeof(R));
+    for (int k = 0; k < 2; k++) B.lS[k] = (R*)take(19 * N * sizeof(R));
     for (int k = 0; k < 2; k++) B.lH[k] = (R*)take(10 * N * sizeof(R));
-    B.lS = (R*)take(19 * N * sizeof(R));
     B.lD = (R*)take(9 * N * sizeof(R));
     B.lJF = (R*)take(3 * N * sizeof(R));
     B.lGeo = (R*)take(25 * N * sizeof(R));
@@ -532,21 +624,20 @@ inline size_t adj_bytes(const cslbm_ctx* c)
 {
     const size_t N = c->N, r = c->r_bytes;
     auto a = [](size_t n) { return (n + 63) / 64 * 64; };
-    return 2 * a(19 * N * r) + 2 * a(10 * N * r) + a(19 * N * r) + a(9 * N * r) + a(3 * N * r) + a(25 * N * r) +
+    return 2 * a(19 * N * r) + 2 * a(10 * N * r) + a(9 * N * r) + a(3 * N * r) + a(25 * N * r) +
            a(9 * N * 8);
 }
 
 unsigned nb(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
-// the boundary rule and pull reversed: lS -> lP[dst], history adjoint in lH[dst]
-template <class R> void finish_step(cslbm_ctx* c, const Lat& L, Bufs<R>& B, int dst)
+// the boundary rule reversed (pass C) on lS[k], lH[k]
+template <class R> void boundary_back(cslbm_ctx* c, const Lat& L, Bufs<R>& B, int k)
 {
     const FaceList f = face_list(c);
     const long long nfc = f.start[f.nseg];
     if (nfc > 0)
         k_adj_boundary<R><<<nb(nfc, 128), 128, 0, c->stream>>>(L, f, (const R*)c->P[c->pc], (const R*)c->H[c->hc],
-                                                               (const R*)c->G[c->gc], B, B.lH[dst]);
-    k_adj_pull<R><<<nb(c->N, 256), 256, 0, c->stream>>>(L, B.lS, B.lP[dst]);
+                                                               (const R*)c->G[c->gc], B.lS[k], B, B.lH[k]);
 }
 
 template <class R> void seed(cslbm_ctx* c, int axis, int side, const double e[3])
@@ -555,7 +646,7 @@ template <class R> void seed(cslbm_ctx* c, int axis, int side, const double e[3]
     Bufs<R> B = bufs<R>(c);
     const int lp = c->adj.lp;
     const size_t N = c->N;
-    cudaMemsetAsync(B.lS, 0, 19 * N * sizeof(R), c->stream);
+    cudaMemsetAsync(B.lS[lp], 0, 19 * N * sizeof(R), c->stream);
     cudaMemsetAsync(B.lH[lp], 0, 10 * N * sizeof(R), c->stream);
     cudaMemsetAsync(B.lGeo, 0, 25 * N * sizeof(R), c->stream);
     cudaMemsetAsync(B.lJ, 0, 9 * N * sizeof(double), c->stream);
@@ -563,8 +654,8 @@ template <class R> void seed(cslbm_ctx* c, int axis, int side, const double e[3]
     const long long nf = (long long)c->n[a1] * c->n[a2];
     k_adj_seed_force<R><<<nb(nf, 128), 128, 0, c->stream>>>(L, (const R*)c->P[c->pc], (const R*)c->H[c->hc],
                                                             (const R*)c->G[c->gc], (const R*)c->J, axis, side, e[0], e[1], e[2],
-                                                            B, B.lH[lp]);
-    finish_step<R>(c, L, B, lp);
+                                                            B.lS[lp], B, B.lH[lp]);
+    boundary_back<R>(c, L, B, lp);
 }
 
 template <class R> void backward(cslbm_ctx* c)
@@ -578,9 +669,16 @@ template <class R> void backward(cslbm_ctx* c)
     const R* H = (const R*)c->H[c->hc];
     const R* geo = (const R*)c->G[c->gc];
     const Mom4<R>* jf = (const Mom4<R>*)c->jf;
-    k_adj_local<R><<<nb(c->N, TB_A), TB_A, 0, c->stream>>>(L, P, H, geo, jf, B.lP[lp], B.lH[lp], B, B.lH[dst]);
-    k_adj_gather<R><<<nb(c->N, 256), 256, 0, c->stream>>>(L, H, geo, jf, B, B.lH[dst]);
-    finish_step<R>(c, L, B, dst);
+    const Plane pl = make_plane(L);
+    const FaceList f = face_list(c);
+    constexpr int TA = kTA<R>;
+    const unsigned nfb = nb(f.start[f.nseg], TA), n01 = (unsigned)c->n[0] * c->n[1];
+    const bool zper = c->p.bc_lo[2] == CSLBM_PERIODIC;
+    const unsigned v0 = zper ? 0 : n01, v1 = zper ? (unsigned)c->N : (unsigned)c->N - n01;
+    k_adj_local<R><<<nfb + nb(v1 - v0, TA), TA, 0, c->stream>>>(L, pl, f, nfb, v0, v1, P, H, geo, jf, B.lS[lp],
+                                                                B.lH[lp], B.lS[dst], B.lH[dst], B);
+    k_adj_gather<R><<<nb(c->N, FB), FB, 0, c->stream>>>(L, pl, H, geo, jf, B.lS[dst], B, B.lH[dst]);
+    boundary_back<R>(c, L, B, dst);
     c->adj.lp = dst;
 }
 
@@ -589,7 +687,7 @@ template <class R> void init_back(cslbm_ctx* c)
     Lat L = make_lat(c);
     Bufs<R> B = bufs<R>(c);
     const int lp = c->adj.lp;
-    k_adj_init<R><<<nb(c->N, 256), 256, 0, c->stream>>>(L, (const R*)c->G[c->gc], B.lP[lp], B.lH[lp], B.lGeo);
+    k_adj_init<R><<<nb(c->N, 128), 128, 0, c->stream>>>(L, (const R*)c->G[c->gc], B.lS[lp], B.lH[lp], B.lGeo);
 }
 
 template <class R> void metric_grad(cslbm_ctx* c, const double* g6, const double* dg18, double* lg6, double* ldg18)
@@ -663,7 +761,7 @@ cslbm_status cslbm_step_backward(cslbm_ctx* c)
     if (cslbm_status s = adj_ready(c)) return s;
     if (c->p.storage == CSLBM_FP64) cslbm::adj::backward<double>(c);
     else cslbm::adj::backward<float>(c);
-    c->launches += 6;
+    c->launches += 5;
     return launched("adjoint step");
 }
 
