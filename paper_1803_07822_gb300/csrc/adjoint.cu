@@ -84,14 +84,12 @@ __device__ __noinline__ void face_inputs(const Lat& L, const R* __restrict__ P, 
                                          int z, R* s, R* d)
 {
     boundary_pops<R, R>(L, P, H, geo, x, y, z, s);
+    R dd[9][3];
+    ghost_differences<R>(L, jf, x, y, z, dd);
 #pragma unroll
-    for (int k = 0; k < 9; k++) {
-        const int l = 2 * k + 1, cx = cvec(l, 0), cy = cvec(l, 1), cz = cvec(l, 2);
-        const Mom4<R> p = mom_site(L, jf, x + cx, y + cy, z + cz), m = mom_site(L, jf, x - cx, y - cy, z - cz);
-        d[3 * k + 0] = p.x - m.x;
-        d[3 * k + 1] = p.y - m.y;
-        d[3 * k + 2] = p.z - m.z;
-    }
+    for (int k = 0; k < 9; k++)
+#pragma unroll
+        for (int i = 0; i < 3; i++) d[3 * k + i] = dd[k][i];
 }
 
 // pass A: threads per block (the staged values of a block fit the static 48 KB)
