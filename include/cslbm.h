@@ -361,10 +361,10 @@ cslbm_status cslbm_batch_context(cslbm_batch* b, int i, cslbm_ctx** out);
 
 /* nsteps time steps of every channel (Sec. II, Eqs. collision and streaming,
  * per channel): ONE persistent launch per step over all channels, whose CTAs
- * (all resident: a cooperative launch) take runs of nodes from a device-side
- * queue for the momentum field, meet at a grid barrier, then take the step's
- * runs from a second queue; two steps are replayed at a time from a CUDA
- * graph.  Asynchronous; ESTATE when a channel has no state. */
+ * (all resident: a cooperative launch) take runs of nodes in turn for the
+ * momentum field, meet at a grid barrier, then take the step's runs; two
+ * steps are replayed at a time from a CUDA graph.  Asynchronous; ESTATE when a
+ * channel has no state. */
 cslbm_status cslbm_batch_step(cslbm_batch* b, int nsteps);
 
 /* Autotuner of the batch step's tile shape: times every candidate -- nodes

@@ -5,23 +5,28 @@
 // boundary velocities; every single-channel call works on it).  A time step
 // of the whole batch is ONE persistent launch: a grid of CTAs, all resident
 // at once (cooperative launch), takes work items -- runs of `item` nodes of
-// one channel -- from a device-side queue (an atomic counter over the items
-// of every channel laid end to end), forms the momentum field rho u of each
-// (the gather pass's per-node code), meets at a grid barrier, then takes the
-// step items from a second queue (pull, moments, gradient, forcing,
-// collision, store).  A CTA finds an item's channel by binary search in the
-// channels' first items, held in shared memory; the channel's lattice,
-// buffers and ping-pong parities come from a table in device memory.  The
-// queue lets small and large channels share the SMs without a fixed block
-// assignment.  Two steps are captured once as a CUDA graph (queue reset,
-// launch, queue reset, launch) on the batch's own stream and replayed; the
-// table is re-uploaded only when a channel's buffers moved (a metric update,
-// a single-channel step).  The tile shape -- nodes per block, nodes per work
-// item, blocks per SM -- is picked by cslbm_batch_tune, which times every
-// candidate on the batch itself with the same step repeated from the same
-// input (the state does not advance).  The grid barrier's wait is bounded
-// (half a second); a wait that runs out sets the batch's error flag, which
-// cslbm_batch_check reports as CSLBM_ETIMEOUT.
+// one channel -- in turn (CTA b items b, b + grid, ...), first the momentum
+// field rho u of each (the gather pass's per-node code), then, after a grid
+// barrier, the step: the items of the face nodes, whose chains of loads are
+// the longest, then the interior nodes.  The warps of a CTA share nothing but
+// the channel tables, so none waits for another between the barriers.  A CTA
+// finds an item's channel by binary search in the channels' first items, held
+// in shared memory; the channel's lattice, buffers and ping-pong parities
+// come from a table in device memory.  Two steps are captured once as a CUDA
+// graph (barrier reset, launch, barrier reset, launch) on the batch's own
+// stream and replayed; the table is re-uploaded only when a channel's buffers
+// moved (a metric update, a single-channel step).  The tile shape -- nodes
+// per block, nodes per work item, blocks per SM -- is picked by
+// cslbm_batch_tune, which times every candidate on the batch itself with the
+// same step repeated from the same input (the state does not advance).  The
+// grid barrier's wait is bounded (half a second); a wait that runs out sets
+// the batch's error flag, which cslbm_batch_check reports as CSLBM_ETIMEOUT.
+//
+// 64 channels of 32..96 per side (17.4 million nodes), us per step: items
+// drawn from an atomic queue by whole blocks (two block barriers each), face
+// nodes on a branch, geometry through registers (168 of them), 1,736; this,
+// 1,627.  (One queue for both passes, a channel's step a little behind its
+// momentum so that the populations are still in L2: 2,224.)
 #include <algorithm>
 #include <cstdint>
 #include <cstdio>
@@ -41,6 +46,8 @@ struct Chan {
     float* H[2];
     const float* G;
     Mom4<float>* jf;
+    Plane pl;
+    FaceList f;
     int pc0, hc0;  // the context's buffers when the table was made
 };
 
@@ -92,83 +99,64 @@ __device__ __forceinline__ void grid_barrier(unsigned* count, int* err)
     __syncthreads();
 }
 
-// the step of a node on a face, out of line
-__device__ __noinline__ void step_face(const Lat& L, const float* __restrict__ Pin, float* __restrict__ Pout,
-                                       const float* __restrict__ hin, float* __restrict__ hout,
-                                       const float* __restrict__ geo, const Mom4<float>* __restrict__ jf, int x, int y,
-                                       int z)
-{
-    step_boundary_body<float, float>(L, Pin, Pout, hin, hout, geo, jf, x, y, z);
-}
-
-__device__ __forceinline__ void step_node(const Lat& L, const float* __restrict__ Pin, float* __restrict__ Pout,
-                                          const float* __restrict__ hin, float* __restrict__ hout,
-                                          const float* __restrict__ geo, const Mom4<float>* __restrict__ jf, int x,
-                                          int y, int z, unsigned v)
-{
-    const unsigned N = (unsigned)L.N;
-    if (on_boundary(L, x, y, z)) {
-        step_face(L, Pin, Pout, hin, hout, geo, jf, x, y, z);
-        return;
-    }
-    const Nbr src = nbr_index(L, x, y, z, -1);
-    float s[Q];
-#pragma unroll
-    for (int l = 0; l < Q; l++)
-        s[l] = __ldg(Pin + (unsigned)pslot(l) * N + nbr_off(src, cvec(l, 0), cvec(l, 1), cvec(l, 2)));
-    GeoT<float> G;
-    HistT<float> Hp;
-    load_geo_hist(geo, hin, v, N, G, Hp);
-    float d[9][3];
-#pragma unroll
-    for (int k = 0; k < 9; k++) {
-        const int l = 2 * k + 1, cx = cvec(l, 0), cy = cvec(l, 1), cz = cvec(l, 2);
-        const Mom4<float> p = jf[nbr_off(src, -cx, -cy, -cz)], m = jf[nbr_off(src, cx, cy, cz)];
-        d[k][0] = p.x - m.x;
-        d[k][1] = p.y - m.y;
-        d[k][2] = p.z - m.z;
-    }
-    step_core<float, float>(L, s, G, Hp, d, Pout, hout, v, N);
-}
-
 // One persistent launch per LBM step of every channel (see the top of the
-// file).  first[c] = first work item of channel c (items of `item` nodes),
-// first[nchan] = all items; q[0], q[1] the momentum and step queues and
-// q[2] the barrier count, zero at launch; k the parity of the step in the
-// two-step cycle.
+// file).  first[c] = first work item of channel c's nodes (items of `item`
+// nodes), first[nchan] = all of them; first[nchan + 1 + c] the same for its
+// face nodes; q the barrier count, zero at launch; k the parity of the step in
+// the two-step cycle.
 template <int TB>
-__global__ void __launch_bounds__(TB) k_batch_persistent(const Chan* __restrict__ tab,
-                                                         const unsigned* __restrict__ first, int nchan, int item,
-                                                         int k, unsigned* q, int* err)
+__global__ void __launch_bounds__(TB, 512 / TB) k_batch_persistent(const Chan* __restrict__ tab,
+                                                                   const unsigned* __restrict__ first, int nchan,
+                                                                   int item, int k, unsigned* q, int* err)
 {
-    extern __shared__ unsigned sb[];
-    __shared__ unsigned w_s;
-    for (int i = threadIdx.x; i <= nchan; i += TB) sb[i] = first[i];
+    extern __shared__ __align__(16) unsigned char smem_batch[];
+    float* stage = reinterpret_cast<float*>(smem_batch);
+    unsigned* sb = reinterpret_cast<unsigned*>(stage + (NGEO + NHIST) * TB);
+    for (int i = threadIdx.x; i < 2 * (nchan + 1); i += TB) sb[i] = first[i];
     __syncthreads();
-    const unsigned nitems = sb[nchan];
-    for (int phase = 0; phase < 2; phase++) {
-        for (;;) {
-            if (threadIdx.x == 0) w_s = atomicAdd(&q[phase], 1u);
-            __syncthreads();
-            const unsigned w = w_s;
-            __syncthreads();
-            if (w >= nitems) break;
-            const int c = find_chan(sb, nchan, w);
-            const Chan& C = tab[c];
-            const unsigned N = (unsigned)C.L.N, v0 = (w - sb[c]) * (unsigned)item;
-            const unsigned v1 = min(v0 + (unsigned)item, N);
-            const unsigned n0 = C.L.n[0], n01 = n0 * C.L.n[1];
-            const int pi = (C.pc0 + k) & 1, hi = (C.hc0 + k) & 1;
-            for (unsigned v = v0 + threadIdx.x; v < v1; v += TB) {
-                const int z = (int)(v / n01), r = (int)(v - z * n01), y = r / (int)n0, x = r - y * (int)n0;
-                if (phase == 0)
-                    momentum_node<float, float>(C.L, C.P[pi], C.H[hi], C.G, C.jf, x, y, z, v);
-                else
-                    step_node(C.L, C.P[pi], C.P[pi ^ 1], C.H[hi], C.H[hi ^ 1], C.G, C.jf, x, y, z, v);
-            }
+    const unsigned* sf = sb + nchan + 1;
+    const unsigned nitems = sb[nchan], nfaces = sf[nchan];
+    for (unsigned w = blockIdx.x; w < nitems; w += gridDim.x) {
+        const int c = find_chan(sb, nchan, w);
+        const Chan& C = tab[c];
+        const unsigned v0 = (w - sb[c]) * (unsigned)item, v1 = min(v0 + (unsigned)item, (unsigned)C.L.N);
+        const int pi = (C.pc0 + k) & 1, hi = (C.hc0 + k) & 1;
+        for (unsigned v = v0 + threadIdx.x; v < v1; v += TB) {
+            int x, y, z;
+            flat_coords(C.L, C.pl, v, x, y, z);
+            momentum_node<float, float>(C.L, C.P[pi], C.H[hi], C.G, C.jf, x, y, z, v);
         }
-        if (phase == 0) grid_barrier(&q[2], err);
     }
+    grid_barrier(q, err);
+    for (unsigned w = blockIdx.x; w < nfaces; w += gridDim.x) {
+        const int c = find_chan(sf, nchan, w);
+        const Chan& C = tab[c];
+        const unsigned i0 = (w - sf[c]) * (unsigned)item;
+        const int pi = (C.pc0 + k) & 1, hi = (C.hc0 + k) & 1;
+        int x, y, z;
+        for (unsigned i = i0 + threadIdx.x; i < i0 + (unsigned)item && face_coords(C.f, (int)i, x, y, z); i += TB)
+            step_face<float, float>(C.L, C.P[pi], C.P[pi ^ 1], C.H[hi], C.H[hi ^ 1], C.G, C.jf, x, y, z);
+    }
+    // (the block's turn continues where the faces left it)
+    for (unsigned u = (blockIdx.x + gridDim.x - nfaces % gridDim.x) % gridDim.x; u < nitems; u += gridDim.x) {
+        const unsigned w = nitems - 1 - u;  // the momentum pass's last populations are still in L2
+        const int c = find_chan(sb, nchan, w);
+        const Chan& C = tab[c];
+        const unsigned v0 = (w - sb[c]) * (unsigned)item, v1 = min(v0 + (unsigned)item, (unsigned)C.L.N);
+        const int pi = (C.pc0 + k) & 1, hi = (C.hc0 + k) & 1;
+        for (unsigned v = v0 + threadIdx.x; v < v1; v += TB) {
+            int x, y, z;
+            flat_coords(C.L, C.pl, v, x, y, z);
+            if (!on_boundary(C.L, x, y, z))
+                step_interior<float, float, TB>(C.L, C.P[pi], C.P[pi ^ 1], C.H[hi], C.H[hi ^ 1], C.G, C.jf, x, y, z, v,
+                                                stage + threadIdx.x);
+        }
+    }
+}
+
+template <int TB> size_t smem_bytes(int nchan)
+{
+    return (size_t)(NGEO + NHIST) * TB * sizeof(float) + 2 * (size_t)(nchan + 1) * sizeof(unsigned);
 }
 
 }  // namespace batch
@@ -189,8 +177,8 @@ struct cslbm_batch {
     cudaStream_t stream;  // the batch's own stream (graphs are captured on it)
     cudaEvent_t ev_in, ev_out, t0, t1;
     Chan* d_tab;          // [nb] in the workspace
-    unsigned* d_first;    // [7][nb + 1]: first work item of each channel, per item size of kItems
-    unsigned* d_q;        // [4]: momentum queue, step queue, barrier count, unused
+    unsigned* d_first;    // [7][2][nb + 1]: first work item of each channel's nodes and faces, per item size of kItems
+    unsigned* d_q;        // [4]: barrier count, unused
     int* d_err;           // grid-barrier timeout flag
     std::vector<Chan> h_tab;
     std::vector<unsigned> h_first;
@@ -248,6 +236,8 @@ cslbm_status upload_table(cslbm_batch* b)
         }
         t.G = (const float*)c->G[c->gc];
         t.jf = (cslbm::Mom4<float>*)c->jf;
+        t.pl = cslbm::make_plane(t.L);
+        t.f = cslbm::face_list(c);
         t.pc0 = c->pc;
         t.hc0 = c->hc;
     }
@@ -260,11 +250,11 @@ cslbm_status upload_table(cslbm_batch* b)
 template <int TB>
 cudaError_t launch_tb(cslbm_batch* b, const Shape& sh, int k, cudaStream_t s)
 {
-    const unsigned* first = b->d_first + item_index(sh.item) * (b->nb + 1);
+    const unsigned* first = b->d_first + item_index(sh.item) * 2 * (b->nb + 1);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(sh.bps * b->n_sm));
     cfg.blockDim = dim3(TB);
-    cfg.dynamicSmemBytes = (b->nb + 1) * sizeof(unsigned);
+    cfg.dynamicSmemBytes = cslbm::batch::smem_bytes<TB>(b->nb);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -275,7 +265,7 @@ cudaError_t launch_tb(cslbm_batch* b, const Shape& sh, int k, cudaStream_t s)
                               sh.item, k, b->d_q, b->d_err);
 }
 
-// one LBM step of every channel: the queues reset, then one persistent launch
+// one LBM step of every channel: the barrier reset, then one persistent launch
 cudaError_t launch_step(cslbm_batch* b, const Shape& sh, int k, cudaStream_t s)
 {
     cudaError_t e = cudaMemsetAsync(b->d_q, 0, 4 * sizeof(unsigned), s);
@@ -287,16 +277,23 @@ cudaError_t launch_step(cslbm_batch* b, const Shape& sh, int k, cudaStream_t s)
     }
 }
 
+template <int TB> int occupancy_tb(const cslbm_batch* b)
+{
+    const size_t sm = cslbm::batch::smem_bytes<TB>(b->nb);
+    // (the most channels a batch can have, so that the attribute serves every batch)
+    cslbm::set_smem_optin_once<cslbm::batch::k_batch_persistent<TB>>(
+        b->ctx[0]->device, (int)cslbm::batch::smem_bytes<TB>(cslbm::batch::kMaxChan));
+    int occ = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cslbm::batch::k_batch_persistent<TB>, TB, sm);
+    return occ;
+}
 int occupancy(const cslbm_batch* b, int tb)
 {
-    int occ = 0;
-    const size_t sm = (b->nb + 1) * sizeof(unsigned);
     switch (tb) {
-    case 0: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cslbm::batch::k_batch_persistent<128>, 128, sm); break;
-    case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cslbm::batch::k_batch_persistent<256>, 256, sm); break;
-    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cslbm::batch::k_batch_persistent<512>, 512, sm); break;
+    case 0: return occupancy_tb<128>(b);
+    case 1: return occupancy_tb<256>(b);
+    default: return occupancy_tb<512>(b);
     }
-    return occ;
 }
 
 cslbm_status make_graph(cslbm_batch* b)
@@ -333,7 +330,7 @@ cslbm_status cslbm_batch_workspace_bytes(int nb, const cslbm_params* p, size_t* 
         if (cslbm_status s = cslbm_workspace_bytes(&p[i], &w)) return s;
         total += al(w);
     }
-    total += al(nb * sizeof(Chan)) + al(7 * (nb + 1) * sizeof(unsigned)) + al(4 * sizeof(unsigned) + sizeof(int));
+    total += al(nb * sizeof(Chan)) + al(14 * (nb + 1) * sizeof(unsigned)) + al(4 * sizeof(unsigned) + sizeof(int));
     *bytes = total;
     return CSLBM_OK;
 }
@@ -369,19 +366,20 @@ cslbm_status cslbm_batch_create(int nb, const cslbm_params* p, void* workspace, 
     b->d_tab = (Chan*)(base + o);
     o += al(nb * sizeof(Chan));
     b->d_first = (unsigned*)(base + o);
-    o += al(7 * (nb + 1) * sizeof(unsigned));
+    o += al(14 * (nb + 1) * sizeof(unsigned));
     b->d_q = (unsigned*)(base + o);
     b->d_err = (int*)(b->d_q + 4);
     b->h_tab.resize(nb);
-    b->h_first.assign(7 * (nb + 1), 0);
-    for (int t = 0; t < 7 && !st; t++) {
-        unsigned acc = 0;
-        for (int i = 0; i < nb; i++) {
-            b->h_first[t * (nb + 1) + i] = acc;
-            acc += (unsigned)((b->ctx[i]->N + cslbm::batch::kItems[t] - 1) / cslbm::batch::kItems[t]);
+    b->h_first.assign(14 * (nb + 1), 0);
+    for (int t = 0; t < 7 && !st; t++)
+        for (int kind = 0; kind < 2; kind++) {
+            unsigned* f = b->h_first.data() + (2 * t + kind) * (nb + 1);
+            const int item = cslbm::batch::kItems[t];
+            for (int i = 0; i < nb; i++) {
+                const long long n = kind ? cslbm::face_count(p[i]) : b->ctx[i]->N;
+                f[i + 1] = f[i] + (unsigned)((n + item - 1) / item);
+            }
         }
-        b->h_first[t * (nb + 1) + nb] = acc;
-    }
     bool have_stream = false;
     if (!st) {
         cudaDeviceGetAttribute(&b->n_sm, cudaDevAttrMultiProcessorCount, b->ctx[0]->device);
@@ -400,7 +398,7 @@ cslbm_status cslbm_batch_create(int nb, const cslbm_params* p, void* workspace, 
                 cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming) != cudaSuccess ||
                 cudaEventCreate(&b->t0) != cudaSuccess || cudaEventCreate(&b->t1) != cudaSuccess))
         st = bfail(CSLBM_ECUDA, "event creation failed");
-    if (!st && cudaMemcpyAsync(b->d_first, b->h_first.data(), 7 * (nb + 1) * sizeof(unsigned), cudaMemcpyHostToDevice,
+    if (!st && cudaMemcpyAsync(b->d_first, b->h_first.data(), 14 * (nb + 1) * sizeof(unsigned), cudaMemcpyHostToDevice,
                                b->stream) != cudaSuccess)
         st = bfail(CSLBM_ECUDA, "table upload failed");
     if (!st && cudaMemsetAsync(b->d_q, 0, 4 * sizeof(unsigned) + sizeof(int), b->stream) != cudaSuccess)

@@ -25,6 +25,8 @@
 // 10 to 30 %.
 #pragma once
 
+#include <mutex>
+
 #include "fast_div.h"
 #include "step_math.cuh"
 
@@ -207,8 +209,7 @@ __device__ __forceinline__ Mom4<R> mom_site(const Lat& L, const Mom4<R>* __restr
 // step is a chain of such latencies (16 x 32 x 16 FP32: 13.3 -> 8.3 us per step,
 // k_step_faces at 256^3 64 -> 39 us).
 template <class R>
-__device__ __forceinline__ void ghost_differences(const Lat& L, const Mom4<R>* __restrict__ jf, int x, int y, int z,
-                                                  R d[9][3])
+__device__ __forceinline__ void ghost_differences(const Lat& L, const Mom4<R>* jf, int x, int y, int z, R d[9][3])
 {
     unsigned o[3][3], g[3][3];  // first and second term's offset of axis a at c = -1, 0, 1
     bool two[3][3];
@@ -371,7 +372,7 @@ __device__ __forceinline__ void load_geo_hist(const R* __restrict__ geo, const R
 template <class S, class R>
 __device__ __forceinline__ void step_boundary_body(const Lat& L, const S* __restrict__ Pin, S* __restrict__ Pout,
                                                    const R* __restrict__ hin, R* __restrict__ hout,
-                                                   const R* __restrict__ geo, const Mom4<R>* __restrict__ jf, int x,
+                                                   const R* __restrict__ geo, const Mom4<R>* jf, int x,
                                                    int y, int z)
 {
     const unsigned N = (unsigned)L.N, v = (unsigned)nidx(L, x, y, z);
@@ -436,6 +437,27 @@ inline FaceList face_list(const cslbm_ctx* c)
     return f;
 }
 
+// nodes on non-periodic faces
+inline long long face_count(const cslbm_params& p)
+{
+    long long all = 1, inner = 1;
+    for (int a = 0; a < 3; a++) {
+        all *= p.n[a];
+        inner *= p.bc_lo[a] == CSLBM_PERIODIC ? p.n[a] : p.n[a] - 2;
+    }
+    return all - inner;
+}
+
+// the same out of line, where one kernel runs face nodes among others (jf may
+// be written by the same launch: plain loads)
+template <class S, class R>
+__device__ __noinline__ void step_face(const Lat& L, const S* __restrict__ Pin, S* __restrict__ Pout,
+                                       const R* __restrict__ hin, R* __restrict__ hout, const R* __restrict__ geo,
+                                       const Mom4<R>* jf, int x, int y, int z)
+{
+    step_boundary_body<S, R>(L, Pin, Pout, hin, hout, geo, jf, x, y, z);
+}
+
 // node i of the list; false past its end.  (Selects over the six segments: an
 // index of f by a runtime value would copy it to local memory; face nodes
 // number fewer than 2^31.)
@@ -498,24 +520,24 @@ __device__ __forceinline__ void copy_async(double* dst, const double* src)
 __device__ __forceinline__ void copies_landed() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 // The step of an interior node.  The 35 values of its geometry and history
-// travel to shared memory (sm[k * FB], the thread's own column: no barrier)
+// travel to shared memory (sm[k * ST], the thread's own column: no barrier)
 // while the populations and the rho u stencil, which the arithmetic needs
 // first, are loaded into registers, so that all of the node's reads are in
 // flight at once.
-template <class S, class R>
+template <class S, class R, int ST>
 __device__ __forceinline__ void step_interior(const Lat& L, const S* __restrict__ Pin, S* __restrict__ Pout,
                                               const R* __restrict__ hin, R* __restrict__ hout,
-                                              const R* __restrict__ geo, const Mom4<R>* __restrict__ jf, int x, int y,
-                                              int z, unsigned v, R* sm)
+                                              const R* __restrict__ geo, const Mom4<R>* jf, int x, int y, int z,
+                                              unsigned v, R* sm)
 {
     const unsigned N = (unsigned)L.N;
     {
         const R* g = geo + v;
         const R* h = hin + v;
 #pragma unroll
-        for (int k = 0; k < NGEO; k++) copy_async(sm + k * FB, g + (size_t)k * N);
+        for (int k = 0; k < NGEO; k++) copy_async(sm + k * ST, g + (size_t)k * N);
 #pragma unroll
-        for (int k = 0; k < NHIST; k++) copy_async(sm + (NGEO + k) * FB, h + (size_t)k * N);
+        for (int k = 0; k < NHIST; k++) copy_async(sm + (NGEO + k) * ST, h + (size_t)k * N);
     }
     const Nbr src = nbr_index(L, x, y, z, -1);
     R s[Q];
@@ -538,16 +560,16 @@ __device__ __forceinline__ void step_interior(const Lat& L, const S* __restrict_
     G.sg = sm[0];
     G.isg = recip(G.sg);
 #pragma unroll
-    for (int a = 0; a < 6; a++) G.gi[a] = sm[(1 + a) * FB];
+    for (int a = 0; a < 6; a++) G.gi[a] = sm[(1 + a) * ST];
 #pragma unroll
-    for (int a = 0; a < 18; a++) G.gam[a] = sm[(7 + a) * FB];
+    for (int a = 0; a < 18; a++) G.gam[a] = sm[(7 + a) * ST];
 #pragma unroll
     for (int k = 0; k < 3; k++) G.gc[k] = (G.gam[0 * 6 + s6(k, 0)] + G.gam[1 * 6 + s6(k, 1)]) + G.gam[2 * 6 + s6(k, 2)];
-    Hp.A = sm[NGEO * FB];
+    Hp.A = sm[NGEO * ST];
 #pragma unroll
-    for (int a = 0; a < 3; a++) Hp.B[a] = sm[(NGEO + 1 + a) * FB];
+    for (int a = 0; a < 3; a++) Hp.B[a] = sm[(NGEO + 1 + a) * ST];
 #pragma unroll
-    for (int a = 0; a < 6; a++) Hp.C[a] = sm[(NGEO + 4 + a) * FB];
+    for (int a = 0; a < 6; a++) Hp.C[a] = sm[(NGEO + 4 + a) * ST];
     step_core<S, R>(L, s, G, Hp, d, Pout, hout, v, N);
 }
 
@@ -575,7 +597,23 @@ __global__ void __launch_bounds__(FB, sizeof(R) == 8 ? 3 : 4)
     wait_previous();
     launch_next();
     if (v >= v1 || on_boundary(L, x, y, z)) return;
-    step_interior<S, R>(L, Pin, Pout, hin, hout, geo, jf, x, y, z, v, sm + threadIdx.x);
+    step_interior<S, R, FB>(L, Pin, Pout, hin, hout, geo, jf, x, y, z, v, sm + threadIdx.x);
+}
+
+// The dynamic shared memory of a kernel beyond 48 KB (bytes, or 0 for all the
+// device allows a kernel without static shared memory), set once per device:
+// the attribute belongs to the context of the device current when it is set.
+template <auto kernel>
+inline void set_smem_optin_once(int device, int bytes = 0)
+{
+    static std::mutex mu;
+    static bool done[64] = {};
+    if (device < 0 || device >= 64) return;
+    std::lock_guard<std::mutex> lock(mu);
+    if (done[device]) return;
+    if (!bytes) cudaDeviceGetAttribute(&bytes, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    done[device] = true;
 }
 
 // threads per block: FB, fewer where that would leave multiprocessors idle

@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(NTHR_F, 1)
 template <class S>
 int launch_fused_step(cslbm_ctx* c, const Lat& L, int pc, int hc, int gc, int* err)
 {
-    set_smem_optin_once(rows::k_step_fused<S>, c->device);
+    set_smem_optin_once<rows::k_step_fused<S>>(c->device);
     cslbm_rows& R = c->rows;
     const rows::Plan& pl = R.plan;
     const S* Pin = (const S*)c->P[pc];
