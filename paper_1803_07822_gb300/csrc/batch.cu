@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(TB, 512 / TB) k_batch_persistent(const Chan* _
 {
     extern __shared__ __align__(16) unsigned char smem_batch[];
     float* stage = reinterpret_cast<float*>(smem_batch);
-    unsigned* sb = reinterpret_cast<unsigned*>(stage + (NGEO + NHIST) * TB);
+    unsigned* sb = reinterpret_cast<unsigned*>(stage + kStaged<float, false> * TB);
     for (int i = threadIdx.x; i < 2 * (nchan + 1); i += TB) sb[i] = first[i];
     __syncthreads();
     const unsigned* sf = sb + nchan + 1;
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(TB, 512 / TB) k_batch_persistent(const Chan* _
             int x, y, z;
             flat_coords(C.L, C.pl, v, x, y, z);
             if (!on_boundary(C.L, x, y, z))
-                step_interior<float, float, TB>(C.L, C.P[pi], C.P[pi ^ 1], C.H[hi], C.H[hi ^ 1], C.G, C.jf, x, y, z, v,
+                step_interior<float, float, TB, false>(C.L, C.P[pi], C.P[pi ^ 1], C.H[hi], C.H[hi ^ 1], C.G, C.jf, x, y, z, v,
                                                 stage + threadIdx.x);
         }
     }
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(TB, 512 / TB) k_batch_persistent(const Chan* _
 
 template <int TB> size_t smem_bytes(int nchan)
 {
-    return (size_t)(NGEO + NHIST) * TB * sizeof(float) + 2 * (size_t)(nchan + 1) * sizeof(unsigned);
+    return (size_t)kStaged<float, false> * TB * sizeof(float) + 2 * (size_t)(nchan + 1) * sizeof(unsigned);
 }
 
 }  // namespace batch

@@ -506,7 +506,7 @@ int launch_faces(const cslbm_ctx* c, const Lat& L, const S* Pin, S* Pout, const 
     return 1;
 }
 
-// asynchronous copy of one value into shared memory
+// asynchronous copy of one value into shared memory (with an L2 policy)
 __device__ __forceinline__ void copy_async(float* dst, const float* src)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
@@ -517,33 +517,65 @@ __device__ __forceinline__ void copy_async(double* dst, const double* src)
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
                  : "memory");
 }
+__device__ __forceinline__ void copy_async(float* dst, const float* src, unsigned long long pol)
+{
+    asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], 4, %2;\n" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(dst)),
+                 "l"(src), "l"(pol)
+                 : "memory");
+}
+__device__ __forceinline__ void copy_async(double* dst, const double* src, unsigned long long pol)
+{
+    asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], 8, %2;\n" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(dst)),
+                 "l"(src), "l"(pol)
+                 : "memory");
+}
 __device__ __forceinline__ void copies_landed() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// The step of an interior node.  The 35 values of its geometry and history
-// travel to shared memory (sm[k * ST], the thread's own column: no barrier)
-// while the populations and the rho u stencil, which the arithmetic needs
-// first, are loaded into registers, so that all of the node's reads are in
-// flight at once.
-template <class S, class R, int ST>
+// values of a node that step_interior stages in shared memory: geometry,
+// history and, on one lattice in FP32, the populations (a copy moves 4 bytes
+// at least, and FP64's would not fit)
+template <class S, bool ONE> constexpr bool kStagePops = ONE && sizeof(S) == 4;
+template <class S, bool ONE> constexpr int kStaged = NGEO + NHIST + (kStagePops<S, ONE> ? Q : 0);
+
+// The step of an interior node.  The staged values travel to shared memory
+// (sm[k * ST], the thread's own column: no barrier) while the rho u stencil
+// loads into registers, so that all of the node's reads are in flight at
+// once.  With ONE (a step of a single lattice) the geometry, read once per
+// step, leaves L2 first and the new populations and history, which the next
+// step reads twice, last: 91 x 77 x 93 FP16 49.0 -> 47.1 us per step, FP32 58.0
+// -> 55.3, 64 x 128 x 64 45.9 -> 43.3; 256^3 the same within 1 %.  In a batch
+// the same costs 2 to 7 % (its channels leave L2 whatever the policy, and the
+// persistent kernel's loops want the shared memory as L1).
+template <class S, class R, int ST, bool ONE>
 __device__ __forceinline__ void step_interior(const Lat& L, const S* __restrict__ Pin, S* __restrict__ Pout,
                                               const R* __restrict__ hin, R* __restrict__ hout,
                                               const R* __restrict__ geo, const Mom4<R>* jf, int x, int y, int z,
                                               unsigned v, R* sm)
 {
+    constexpr bool POPS = kStagePops<S, ONE>;
     const unsigned N = (unsigned)L.N;
     {
         const R* g = geo + v;
         const R* h = hin + v;
+        const unsigned long long once = ONE ? policy_evict_first() : 0;
 #pragma unroll
-        for (int k = 0; k < NGEO; k++) copy_async(sm + k * ST, g + (size_t)k * N);
+        for (int k = 0; k < NGEO; k++) {
+            if constexpr (ONE) copy_async(sm + k * ST, g + (size_t)k * N, once);
+            else copy_async(sm + k * ST, g + (size_t)k * N);
+        }
 #pragma unroll
         for (int k = 0; k < NHIST; k++) copy_async(sm + (NGEO + k) * ST, h + (size_t)k * N);
     }
     const Nbr src = nbr_index(L, x, y, z, -1);
     R s[Q];
 #pragma unroll
-    for (int l = 0; l < Q; l++)
-        s[l] = R(Store<S>::ld(Pin + (unsigned)pslot(l) * N + nbr_off(src, cvec(l, 0), cvec(l, 1), cvec(l, 2))));
+    for (int l = 0; l < Q; l++) {
+        const S* p = Pin + (unsigned)pslot(l) * N + nbr_off(src, cvec(l, 0), cvec(l, 1), cvec(l, 2));
+        if constexpr (POPS) copy_async(sm + (NGEO + NHIST + l) * ST, p);
+        else s[l] = R(Store<S>::ld(p));
+    }
     R d[9][3];
 #pragma unroll
     for (int k = 0; k < 9; k++) {
@@ -555,6 +587,10 @@ __device__ __forceinline__ void step_interior(const Lat& L, const S* __restrict_
         d[k][2] = p.z - m.z;
     }
     copies_landed();
+    if constexpr (POPS) {
+#pragma unroll
+        for (int l = 0; l < Q; l++) s[l] = sm[(NGEO + NHIST + l) * ST];
+    }
     GeoT<R> G;
     HistT<R> Hp;
     G.sg = sm[0];
@@ -570,7 +606,7 @@ __device__ __forceinline__ void step_interior(const Lat& L, const S* __restrict_
     for (int a = 0; a < 3; a++) Hp.B[a] = sm[(NGEO + 1 + a) * ST];
 #pragma unroll
     for (int a = 0; a < 6; a++) Hp.C[a] = sm[(NGEO + 4 + a) * ST];
-    step_core<S, R>(L, s, G, Hp, d, Pout, hout, v, N);
+    step_core<S, R, ONE>(L, s, G, Hp, d, Pout, hout, v, N, ONE ? policy_evict_last() : 0);
 }
 
 // The step of every node: the first nfb blocks take the face nodes (the
@@ -583,7 +619,7 @@ __global__ void __launch_bounds__(FB, sizeof(R) == 8 ? 3 : 4)
                 const R* __restrict__ hin, R* __restrict__ hout, const R* __restrict__ geo,
                 const Mom4<R>* __restrict__ jf)
 {
-    __shared__ R sm[(NGEO + NHIST) * FB];
+    __shared__ R sm[kStaged<S, true> * FB];
     int x, y, z;
     if (blockIdx.x < nfb) {
         const bool ok = face_coords(f, (int)(blockIdx.x * blockDim.x + threadIdx.x), x, y, z);
@@ -597,7 +633,7 @@ __global__ void __launch_bounds__(FB, sizeof(R) == 8 ? 3 : 4)
     wait_previous();
     launch_next();
     if (v >= v1 || on_boundary(L, x, y, z)) return;
-    step_interior<S, R, FB>(L, Pin, Pout, hin, hout, geo, jf, x, y, z, v, sm + threadIdx.x);
+    step_interior<S, R, FB, true>(L, Pin, Pout, hin, hout, geo, jf, x, y, z, v, sm + threadIdx.x);
 }
 
 // The dynamic shared memory of a kernel beyond 48 KB (bytes, or 0 for all the
