@@ -4,6 +4,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 
 #include "ctx.h"
@@ -179,6 +180,68 @@ cslbm_status read_scratch(cslbm_ctx* c, double* out, int k)
     return CSLBM_OK;
 }
 
+// Mapped host memory the reductions write their result to: 64 slots of four
+// doubles in one page of the process, taken by a context's first reduction and
+// given back by cslbm_destroy (a context without one copies its result).
+constexpr int kSlots = 64;
+std::mutex g_slot_mu;
+double* g_slot_page = nullptr;
+unsigned long long g_slot_used = 0;
+
+double* slot_take()
+{
+    std::lock_guard<std::mutex> lock(g_slot_mu);
+    if (!g_slot_page) {
+        // (another thread may be capturing a stream)
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        void* p = nullptr;
+        void* d = nullptr;
+        if (cudaHostAlloc(&p, kSlots * 4 * sizeof(double), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess) {
+            if (cudaHostGetDevicePointer(&d, p, 0) == cudaSuccess && d == p) g_slot_page = (double*)p;
+            else cudaFreeHost(p);
+        }
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        cudaGetLastError();
+        if (!g_slot_page) return nullptr;
+    }
+    for (int i = 0; i < kSlots; i++)
+        if (!(g_slot_used >> i & 1)) {
+            g_slot_used |= 1ull << i;
+            return g_slot_page + 4 * i;
+        }
+    return nullptr;
+}
+void slot_give(double* s)
+{
+    if (!s) return;
+    std::lock_guard<std::mutex> lock(g_slot_mu);
+    g_slot_used &= ~(1ull << ((s - g_slot_page) / 4));
+}
+
+// k sums of a reduction launched by run(acc, host): through the context's
+// slot, else through the scratch with a copy
+template <class F> cslbm_status reduce(cslbm_ctx* c, double* out, int k, const char* what, F run)
+{
+    if (!c->slot_tried) {
+        c->slot = slot_take();
+        c->slot_tried = 1;
+    }
+    double* acc = c->scratch + 8;  // zero between reductions
+    run(acc, c->slot);
+    c->launches++;
+    LAUNCH_CHECK(what);
+    if (c->slot) {
+        CUDA_TRY(cudaStreamSynchronize(c->stream));
+        for (int i = 0; i < k; i++) out[i] = ((volatile double*)c->slot)[i];
+        return CSLBM_OK;
+    }
+    CUDA_TRY(cudaMemcpyAsync(out, acc, k * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(cudaMemsetAsync(acc, 0, 8 * sizeof(double), c->stream));
+    CUDA_TRY(cudaStreamSynchronize(c->stream));
+    return CSLBM_OK;
+}
+
 cslbm_status metric_flag(cslbm_ctx* c)
 {
     int hbad = 0;
@@ -340,6 +403,8 @@ cslbm_status cslbm_create(const cslbm_params* p, void* ws, size_t bytes, void* s
         c->face_n[k] = L.face_n[k];
     }
     c->scratch = (double*)(b + L.off_scratch);
+    c->slot = nullptr;
+    c->slot_tried = 0;
     c->rows.done = (unsigned*)(b + L.off_done);
     c->staging = (double*)(b + L.off_staging);
     c->chunk = L.chunk;
@@ -371,6 +436,7 @@ cslbm_status cslbm_destroy(cslbm_ctx* c)
     if (!c) return fail(CSLBM_EINVAL, "ctx is null");
     cudaStreamSynchronize(c->stream);
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
+    slot_give(c->slot);
     delete c;
     return CSLBM_OK;
 }
@@ -587,22 +653,15 @@ cslbm_status cslbm_total_mass(cslbm_ctx* c, double* out)
 {
     if (!c || !out) return fail(CSLBM_EINVAL, "null argument");
     if (!c->has_state) return fail(CSLBM_ESTATE, "no state");
-    CUDA_TRY(cudaMemsetAsync(c->scratch, 0, 8 * sizeof(double), c->stream));
-    c->ops->mass(c, c->scratch);
-    c->launches++;
-    LAUNCH_CHECK("mass kernel");
-    return read_scratch(c, out, 1);
+    return reduce(c, out, 1, "mass kernel", [&](double* acc, double* host) { c->ops->mass(c, acc, host); });
 }
 
 cslbm_status cslbm_wall_force(cslbm_ctx* c, int axis, int side, double out3[3])
 {
     if (!c || !out3 || axis < 0 || axis > 2 || side < 0 || side > 1) return fail(CSLBM_EINVAL, "bad argument");
     if (!c->has_state) return fail(CSLBM_ESTATE, "no state");
-    CUDA_TRY(cudaMemsetAsync(c->scratch, 0, 8 * sizeof(double), c->stream));
-    c->ops->wall_force(c, axis, side, c->scratch);
-    c->launches++;
-    LAUNCH_CHECK("wall-force kernel");
-    return read_scratch(c, out3, 3);
+    return reduce(c, out3, 3, "wall-force kernel",
+                  [&](double* acc, double* host) { c->ops->wall_force(c, axis, side, acc, host); });
 }
 
 cslbm_status cslbm_check(cslbm_ctx* c)

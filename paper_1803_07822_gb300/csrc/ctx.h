@@ -55,6 +55,8 @@ struct cslbm_ctx {
     double* face[6]; // [3][face nodes] boundary velocity of non-periodic faces
     long long face_n[6];
     double* scratch; // 64 doubles of reduction space
+    double* slot;    // four doubles of mapped host memory for reduced values, or null
+    int slot_tried;
     double* staging; // host-transfer staging, chunk * 24 doubles
     long long chunk; // nodes per staging chunk
     int pc, hc, gc;  // current buffer of P, H, G
@@ -108,10 +110,11 @@ struct cslbm_ops {
     // rho, u (or v) of nodes [v0, v0+cnt) into out arrays with the given stride
     void (*readout)(const cslbm_ctx*, double* rho, double* u3, long long stride, long long v0,
                     long long cnt, int cartesian);
-    // scratch[0] += sum sqrt(g) rho
-    void (*mass)(const cslbm_ctx*, double* acc);
-    // acc[0..2] += wall force of face (axis, side)
-    void (*wall_force)(const cslbm_ctx*, int axis, int side, double* acc);
+    // acc[0] += sum sqrt(g) rho; with `host` (mapped host memory) the sum goes
+    // there instead and acc stays zero
+    void (*mass)(const cslbm_ctx*, double* acc, double* host);
+    // acc[0..2] += wall force of face (axis, side); `host` as above
+    void (*wall_force)(const cslbm_ctx*, int axis, int side, double* acc, double* host);
     // acc[0] += number of unstable nodes
     void (*check)(const cslbm_ctx*, double* acc);
 };

@@ -834,11 +834,16 @@ __global__ void __launch_bounds__(TPB, 4) k_readout(const __grid_constant__ Lat 
     }
 }
 
-// FP64 block reduction of up to 3 values, one atomic per block and value.
-template <int K>
-__device__ __forceinline__ void block_reduce_add(double (&val)[K], double* acc)
+// FP64 block reduction of up to 3 values over NT threads, one atomic per
+// block and value onto acc.  With `host` (mapped host memory) the last block
+// to add moves the sums there and leaves acc and its ticket (the 8th value of
+// acc) zero for the next call, so that a reduction is one launch: clearing
+// acc and copying it to pageable memory around it cost a coupled loop about
+// 8 us per reduction (32 x 32 x 64, two per step: 709 -> 625 us for five steps).
+template <int K, int NT>
+__device__ __forceinline__ void block_reduce_add(double (&val)[K], double* acc, double* host = nullptr)
 {
-    __shared__ double part[K][TPB / 32];
+    __shared__ double part[K][NT / 32];
 #pragma unroll
     for (int k = 0; k < K; k++)
 #pragma unroll
@@ -851,10 +856,19 @@ __device__ __forceinline__ void block_reduce_add(double (&val)[K], double* acc)
     if (wid == 0) {
 #pragma unroll
         for (int k = 0; k < K; k++) {
-            double s = lane < (TPB / 32) ? part[k][lane] : 0.0;
+            double s = lane < (NT / 32) ? part[k][lane] : 0.0;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
             if (lane == 0) atomicAdd(acc + k, s);
+        }
+        if (lane == 0 && host) {
+            __threadfence();
+            if (atomicInc((unsigned*)(acc + 7), gridDim.x - 1) == gridDim.x - 1) {
+                __threadfence();
+#pragma unroll
+                for (int k = 0; k < K; k++)
+                    host[k] = __longlong_as_double((long long)atomicExch((unsigned long long*)(acc + k), 0ull));
+            }
         }
     }
 }
@@ -880,7 +894,7 @@ __device__ __forceinline__ double exact64(double v) { return v; }
 // one multiply and one add.
 template <class S, class R>
 __global__ void __launch_bounds__(TPB, 3) k_mass(Lat L, const S* __restrict__ P, const R* __restrict__ hist,
-                                              const R* __restrict__ geo, double* acc)
+                                              const R* __restrict__ geo, double* acc, double* host)
 {
     double val[1] = {0.0};
     const unsigned N = (unsigned)L.N, n0 = L.n[0], n1 = L.n[1];
@@ -900,13 +914,14 @@ __global__ void __launch_bounds__(TPB, 3) k_mass(Lat L, const S* __restrict__ P,
         }
         val[0] += exact64(sg) * exact64(rho);
     }
-    block_reduce_add<1>(val, acc);
+    block_reduce_add<1, TPB>(val, acc, host);
 }
 
+constexpr int TPW = 128;  // threads of a wall-force block
 template <class S, class R>
-__global__ void __launch_bounds__(TPB) k_wall_force(Lat L, const S* __restrict__ P, const R* __restrict__ hist,
+__global__ void __launch_bounds__(TPW) k_wall_force(const __grid_constant__ Lat L, const S* __restrict__ P, const R* __restrict__ hist,
                                                     const R* __restrict__ geo, const R* __restrict__ J,
-                                                    int axis, int side, double* acc)
+                                                    int axis, int side, double* acc, double* host)
 {
     // one thread per node of the face
     const int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
@@ -941,7 +956,7 @@ __global__ void __launch_bounds__(TPB) k_wall_force(Lat L, const S* __restrict__
             val[a] = sgn * s * double(G.sg);
         }
     }
-    block_reduce_add<3>(val, acc);
+    block_reduce_add<3, TPW>(val, acc, host);
 }
 
 template <class S, class R>
@@ -967,7 +982,7 @@ __global__ void __launch_bounds__(TPB) k_check(Lat L, const S* __restrict__ P, c
         const bool bad = !(double(M.rho) > 0.0) || !(s2 <= 0.09);  // false for NaN too
         val[0] = bad ? 1.0 : 0.0;
     }
-    block_reduce_add<1>(val, acc);
+    block_reduce_add<1, TPB>(val, acc);
 }
 
 
@@ -1057,19 +1072,19 @@ template <class S, class R> struct Launch {
         k_readout<S, R><<<nblocks(cnt), TPB, 0, c->stream>>>(make_lat(c), P(c, c->pc), H(c, c->hc), G(c, c->gc), (const R*)c->J,
                                                              rho, u3, stride, v0, cnt, cartesian);
     }
-    static void mass(const cslbm_ctx* c, double* acc)
+    static void mass(const cslbm_ctx* c, double* acc, double* host)
     {
         // resident blocks of TPB threads: three per SM at the kernel's register bound
         const unsigned nb = nblocks(c->N), res = 3u * (unsigned)c->n_sm;
         k_mass<S, R><<<nb < res ? nb : res, TPB, 0, c->stream>>>(make_lat(c), P(c, c->pc), H(c, c->hc), G(c, c->gc),
-                                                                acc);
+                                                                acc, host);
     }
-    static void wall_force(const cslbm_ctx* c, int axis, int side, double* acc)
+    static void wall_force(const cslbm_ctx* c, int axis, int side, double* acc, double* host)
     {
         const int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
         long long nf = (long long)c->n[a1] * c->n[a2];
-        k_wall_force<S, R><<<nblocks(nf), TPB, 0, c->stream>>>(make_lat(c), P(c, c->pc), H(c, c->hc), G(c, c->gc),
-                                                               (const R*)c->J, axis, side, acc);
+        k_wall_force<S, R><<<(unsigned)((nf + TPW - 1) / TPW), TPW, 0, c->stream>>>(make_lat(c), P(c, c->pc), H(c, c->hc), G(c, c->gc),
+                                                               (const R*)c->J, axis, side, acc, host);
     }
     static void check(const cslbm_ctx* c, double* acc)
     {
