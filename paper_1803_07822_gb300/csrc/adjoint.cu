@@ -29,16 +29,16 @@
 // Pass A is bound by the latency of its loads (about 700 B per node at 128
 // registers), so the 89 values of a node that the arithmetic needs late --
 // geometry, histories, the gathered lS, the geometry adjoint -- travel to
-// shared memory asynchronously and face nodes run in blocks of their own; B
-// reads the 90 lD values of a node's neighbours without a face test (lD of a
-// face node is zero).  64 x 128 x 64 FP32, us per backward step: A 175 -> 112,
-// the pull of a pass of its own 29 -> 0.
+// shared memory asynchronously and face nodes run in blocks of their own.
+// 64 x 128 x 64 FP32, us per backward step: A 175 -> 87,
+// the pull of a pass of its own 29 -> 0 (B below).
 #include <cstdio>
 #include <string>
 
 #include "ctx.h"
 #include "make_lat.h"
 #include "adjoint.cuh"
+#include "march_tiles.cuh"
 
 namespace cslbm {
 namespace adj {
@@ -277,96 +277,126 @@ __global__ void __launch_bounds__(kTA<R>, 4)
         for (int i = 0; i < 3; i++) B.lD[(k * 3 + i) * N + v] = lD[k][i];
 }
 
-// pass B: the rho-u adjoint of a face node gathered (neighbours past a face are none)
+// pass B: the rho-u adjoint of node y is, by the antisymmetry of the stencil,
+// lj_i = -sum_k G_k(lD_ki) with lD zero beyond a face, so the factored sums of
+// the lattice gradient serve (lattice_deriv.cu): blocks march along axis 2
+// with the nine lD planes of a 32 x 8 tile and its rim in shared memory.  (One
+// thread per node read 90 lD values of its neighbours: 64 -> 48 us on 64 x 128
+// x 64 FP32; 66 at three blocks per SM, which spills.)  In units of 1/12, with d_x = X(x + 1) - X(x - 1) of X = lD_0i, d_y
+// of Y = lD_1i and q = 2 Z + Z(x +- 1) + Z(y +- 1) of Z = lD_2i:
+//   -12 lj_i = 2 (d_x + d_y) + d_x(y +- 1) + d_y(x +- 1) + (d_x + d_y)(z +- 1) + q(z + 1) - q(z - 1).
 template <class R>
-__device__ __noinline__ Mom4<R> gather_face(const Lat& L, const R* __restrict__ lD, int x, int y, int z)
-{
-    const size_t N = L.N;
-    R lj[3] = {R(0), R(0), R(0)};
-#pragma unroll
-    for (int l = 1; l < Q; l++) {
-        const int c[3] = {cvec(l, 0), cvec(l, 1), cvec(l, 2)};
-        int r[3] = {x - c[0], y - c[1], z - c[2]};
-        bool ok = true;
-#pragma unroll
-        for (int a = 0; a < 3; a++)
-            if (r[a] < 0 || r[a] >= L.n[a]) {
-                if ((r[a] < 0 ? L.bclo[a] : L.bchi[a]) == BC_PERIODIC) r[a] = wrapc(r[a], L.n[a]);
-                else ok = false;
-            }
-        if (!ok) continue;
-        const unsigned u = (unsigned)nidx(L, r[0], r[1], r[2]);
-        const R w = R(3.0 * wq(l));
-#pragma unroll
-        for (int k = 0; k < 3; k++) {
-            if (!c[k]) continue;
-#pragma unroll
-            for (int i = 0; i < 3; i++) lj[i] += w * R(c[k]) * lD[(k * 3 + i) * N + u];
-        }
-    }
-    return Mom4<R>{lj[0], lj[1], lj[2], R(0)};
-}
-
-template <class R>
-__global__ void __launch_bounds__(FB, sizeof(R) == 8 ? 4 : 8)
-    k_adj_gather(const __grid_constant__ Lat L, const __grid_constant__ Plane pl, const R* __restrict__ H,
+__global__ void __launch_bounds__(TX* TY, sizeof(R) == 8 ? 1 : 2)
+    k_adj_gather(const __grid_constant__ Lat L, const __grid_constant__ Tiles T, const R* __restrict__ H,
                  const R* __restrict__ geo, const Mom4<R>* __restrict__ jf, R* __restrict__ lS,
                  const __grid_constant__ Bufs<R> B, R* __restrict__ lHi)
 {
-    const unsigned v = blockIdx.x * FB + threadIdx.x;
-    if (v >= (unsigned)L.N) return;
+    __shared__ R fs[9][TY + 2][TX + 2], dxs[3][TY + 2][TX], dys[3][TY][TX + 2];
+    const int tx = threadIdx.x, ty = threadIdx.y, t = ty * TX + tx;
+    int x0, y0, za, zb;
+    tile_of(T, 0, 0, x0, y0, za, zb);
+    const int x = x0 + tx, y = y0 + ty, n0 = L.n[0], n1 = L.n[1], n2 = L.n[2];
+    const bool mine = x < n0 && y < n1;
     const size_t N = L.N;
-    int x, y, z;
-    flat_coords(L, pl, v, x, y, z);
-    R lj[3];
-    if (on_boundary(L, x, y, z)) {
-        const Mom4<R> g = gather_face<R>(L, B.lD, x, y, z);
-        lj[0] = g.x;
-        lj[1] = g.y;
-        lj[2] = g.z;
-    } else {
-        // interior nodes x' = y - c whose stencil site x' + c is this node
-        const Nbr src = nbr_index(L, x, y, z, -1);
-        const R* lD = B.lD;
-        R face[3] = {R(0), R(0), R(0)}, edge[3] = {R(0), R(0), R(0)};
+    // the tile's entries this thread loads: in-plane offset, or -1 where a face cuts them off (zero)
+    int off[2];
 #pragma unroll
-        for (int l = 1; l < Q; l++) {
-            const int c[3] = {cvec(l, 0), cvec(l, 1), cvec(l, 2)};
-            const unsigned u = nbr_off(src, c[0], c[1], c[2]);
+    for (int k = 0; k < 2; k++) {
+        const int i = t + k * TX * TY, ly = i / (TX + 2), lx = i - ly * (TX + 2);
+        int r0 = x0 - 1 + lx, r1 = y0 - 1 + ly;
+        bool ok = i < (TX + 2) * (TY + 2) && r0 <= n0 && r1 <= n1;
+        if (r0 < 0 || r0 >= n0) {
+            ok = ok && L.bclo[0] == BC_PERIODIC;
+            r0 = wrapc(r0, n0);
+        }
+        if (r1 < 0 || r1 >= n1) {
+            ok = ok && L.bclo[1] == BC_PERIODIC;
+            r1 = wrapc(r1, n1);
+        }
+        off[k] = ok ? r1 * n0 + r0 : -1;
+        if (!ok && i < (TX + 2) * (TY + 2))
 #pragma unroll
-            for (int k = 0; k < 3; k++) {
-                if (!c[k]) continue;
+            for (int q = 0; q < 9; q++) (&fs[q][0][0])[i] = R(0);
+    }
+    const unsigned n01 = (unsigned)n0 * n1;
+    R na[3], nb_[3], mb[3], qa[3], qb[3];
 #pragma unroll
-                for (int i = 0; i < 3; i++) {
-                    const R t = lD[(k * 3 + i) * N + u];
-                    if (l <= 6) face[i] += c[k] > 0 ? t : -t;
-                    else edge[i] += c[k] > 0 ? t : -t;
+    for (int i = 0; i < 3; i++) na[i] = nb_[i] = mb[i] = qa[i] = qb[i] = R(0);
+    for (int p = za - 1; p <= zb; p++) {
+        int pz = p;
+        if (p < 0 || p >= n2) pz = L.bclo[2] == BC_PERIODIC ? wrapc(p, n2) : -1;
+        R nn[3], m[3], q[3];
+        if (pz >= 0) {
+            const R* f = B.lD + (size_t)pz * n01;
+#pragma unroll
+            for (int k = 0; k < 2; k++)
+                if (off[k] >= 0)
+#pragma unroll
+                    for (int c = 0; c < 9; c++) (&fs[c][0][0])[t + k * TX * TY] = __ldg(f + c * N + off[k]);
+            __syncthreads();
+            R dx[3], dy[3];
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+                const R(*X)[TX + 2] = fs[i];
+                const R(*Y)[TX + 2] = fs[3 + i];
+                const R(*Z)[TX + 2] = fs[6 + i];
+                dx[i] = X[ty + 1][tx + 2] - X[ty + 1][tx];
+                dy[i] = Y[ty + 2][tx + 1] - Y[ty][tx + 1];
+                q[i] = fmad(R(2), Z[ty + 1][tx + 1],
+                            (Z[ty + 1][tx + 2] + Z[ty + 1][tx]) + (Z[ty + 2][tx + 1] + Z[ty][tx + 1]));
+                dxs[i][ty + 1][tx] = dx[i];
+                dys[i][ty][tx + 1] = dy[i];
+                // the rims: d_x of the rows beside the tile, d_y of the columns
+                if (ty < 2) dxs[i][ty * (TY + 1)][tx] = X[ty * (TY + 1)][tx + 2] - X[ty * (TY + 1)][tx];
+                else if (ty == 2 && tx < 2 * TY) {
+                    const int r = tx >> 1, col = (tx & 1) * (TX + 1);
+                    dys[i][r][col] = Y[r + 2][col] - Y[r][col];
                 }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+                nn[i] = dx[i] + dy[i];
+                m[i] = fmad(R(2), nn[i], (dxs[i][ty][tx] + dxs[i][ty + 2][tx]) + (dys[i][ty][tx] + dys[i][ty][tx + 2]));
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 3; i++) nn[i] = m[i] = q[i] = R(0);
+        }
+        if (p > za && mine) {
+            const unsigned v = (unsigned)(p - 1) * n01 + (unsigned)y * n0 + x;
+            R ls[Q], lj[3];
+#pragma unroll
+            for (int l = 1; l < Q; l++) ls[l] = lS[l * N + v];
+            // j(y) = sqrt(g) m1 + B/2 with m1 = (j - B/2) / sqrt(g)
+            const R sg = geo[v], isg = recip(sg);
+            const Mom4<R> jv = jf[v];
+            const R jj[3] = {jv.x, jv.y, jv.z};
+            R lsg = R(0);
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+                lj[i] = fmad(R(-1.0 / 12.0), mb[i] + (na[i] + nn[i]) + (q[i] - qa[i]), B.lJF[i * N + v]);
+                const R Bh = H[(1 + i) * N + v];
+                lsg += (jj[i] - R(0.5) * Bh) * isg * lj[i];
+                lHi[(1 + i) * N + v] += R(0.5) * lj[i];
+            }
+            B.lGeo[v] += lsg;
+#pragma unroll
+            for (int l = 1; l < Q; l++) {
+                R u = R(0);
+#pragma unroll
+                for (int a = 0; a < 3; a++) u += R(cvec(l, a)) * lj[a];
+                lS[l * N + v] = ls[l] + sg * u;
             }
         }
 #pragma unroll
-        for (int i = 0; i < 3; i++) lj[i] = fmad(R(1.0 / 6.0), face[i], R(1.0 / 12.0) * edge[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < 3; i++) lj[i] += B.lJF[i * N + v];
-    // j(y) = sqrt(g) m1 + B/2 with m1 = (j - B/2) / sqrt(g)
-    const R sg = geo[v], isg = recip(sg);
-    const Mom4<R> jv = jf[v];
-    const R jj[3] = {jv.x, jv.y, jv.z};
-    R lsg = R(0);
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        const R Bh = H[(1 + a) * N + v];
-        lsg += (jj[a] - R(0.5) * Bh) * isg * lj[a];
-        lHi[(1 + a) * N + v] += R(0.5) * lj[a];
-    }
-    B.lGeo[v] += lsg;
-#pragma unroll
-    for (int l = 1; l < Q; l++) {
-        R t = R(0);
-#pragma unroll
-        for (int a = 0; a < 3; a++) t += R(cvec(l, a)) * lj[a];
-        lS[l * N + v] += sg * t;
+        for (int i = 0; i < 3; i++) {
+            na[i] = nb_[i];
+            nb_[i] = nn[i];
+            mb[i] = m[i];
+            qa[i] = qb[i];
+            qb[i] = q[i];
+        }
     }
 }
 
@@ -675,7 +705,8 @@ template <class R> void backward(cslbm_ctx* c)
     const unsigned v0 = zper ? 0 : n01, v1 = zper ? (unsigned)c->N : (unsigned)c->N - n01;
     k_adj_local<R><<<nfb + nb(v1 - v0, TA), TA, 0, c->stream>>>(L, pl, f, nfb, v0, v1, P, H, geo, jf, B.lS[lp],
                                                                 B.lH[lp], B.lS[dst], B.lH[dst], B);
-    k_adj_gather<R><<<nb(c->N, FB), FB, 0, c->stream>>>(L, pl, H, geo, jf, B.lS[dst], B, B.lH[dst]);
+    const Tiles T = tiles_of(c->n_sm, c->n[0], c->n[1], 0, c->n[2], 1);
+    k_adj_gather<R><<<tile_grid(T, 1), dim3(TX, TY), 0, c->stream>>>(L, T, H, geo, jf, B.lS[dst], B, B.lH[dst]);
     boundary_back<R>(c, L, B, dst);
     c->adj.lp = dst;
 }

@@ -25,6 +25,7 @@
 
 #include "ctx.h"
 #include "lbm_device.cuh"
+#include "march_tiles.cuh"
 
 cslbm_status cslbm_record_error(cslbm_status s, const char* msg);
 
@@ -150,21 +151,6 @@ __device__ __noinline__ double correct_far(const Box& B, const double* __restric
         else se += fl;
     }
     return fma(5.0 / 3.0, f0, -fma(0.5, se, sf) * (1.0 / 18.0));
-}
-
-// Tiles of the marching kernels: TX x TY columns, one thread each, by a chunk
-// of planes; the block index counts tiles along axis 0, then 1, then chunks.
-constexpr int TX = 32, TY = 8;
-struct Tiles {
-    int nx, ny, chunk, first, last;  // planes first .. last - 1 in chunks of `chunk`
-};
-__device__ __forceinline__ void tile_of(const Tiles& T, int lo0, int lo1, int& x0, int& y0, int& za, int& zb)
-{
-    const int b = blockIdx.x, bx = b % T.nx, r = b / T.nx, by = r % T.ny, bz = r / T.ny;
-    x0 = lo0 + bx * TX;
-    y0 = lo1 + by * TY;
-    za = T.first + bz * T.chunk;
-    zb = min(T.last, za + T.chunk);
 }
 
 // Order 4: F / 12 on the padded lattice.  With the in-plane sums q = s_x + s_y
@@ -353,25 +339,6 @@ bool device_memory(const void* p)
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-// Chunks of at most 32 planes (a march repeats two planes of its neighbours'),
-// shorter ones while there are fewer than eight blocks per SM
-Tiles tiles_of(const cslbm_ctx* c, int e0, int e1, int first, int last, int ncomp)
-{
-    Tiles T;
-    T.nx = (e0 + TX - 1) / TX;
-    T.ny = (e1 + TY - 1) / TY;
-    T.first = first;
-    T.last = last;
-    T.chunk = 32;
-    while (T.chunk > 4 && (long long)T.nx * T.ny * ncomp * ((last - first + T.chunk - 1) / T.chunk) < 8LL * c->n_sm)
-        T.chunk /= 2;
-    return T;
-}
-dim3 tile_grid(const Tiles& T, int ncomp)
-{
-    return dim3((unsigned)T.nx * T.ny * ((T.last - T.first + T.chunk - 1) / T.chunk), (unsigned)ncomp);
-}
-
 size_t pad_bytes(const cslbm_ctx* c, int ncomp, int order)
 {
     return (size_t)ncomp * (size_t)box_of(c, order).Ne * sizeof(double);
@@ -388,12 +355,12 @@ cslbm_status gradient(cslbm_ctx* c, const double* f, int ncomp, int order, doubl
     const Box B = box_of(c, order);
     double* F = (double*)scratch;
     if (order == 4) {
-        const Tiles T = tiles_of(c, B.ne[0], B.ne[1], -B.pad[2], B.n[2] + B.pad[2], ncomp);
+        const Tiles T = tiles_of(c->n_sm, B.ne[0], B.ne[1], -B.pad[2], B.n[2] + B.pad[2], ncomp);
         k_correct<<<tile_grid(T, ncomp), dim3(TX, TY), 0, c->stream>>>(B, T, f, F);
     } else {
         k_pad<<<dim3((unsigned)((B.Ne + TBL - 1) / TBL), (unsigned)ncomp), TBL, 0, c->stream>>>(B, f, F);
     }
-    const Tiles T = tiles_of(c, B.n[0], B.n[1], 0, B.n[2], ncomp);
+    const Tiles T = tiles_of(c->n_sm, B.n[0], B.n[1], 0, B.n[2], ncomp);
     k_grad<<<tile_grid(T, ncomp), dim3(TX, TY), 0, c->stream>>>(B, T, ncomp, F, out);
     c->launches += 2;
     const cudaError_t e = cudaGetLastError();
