@@ -207,6 +207,16 @@ cslbm_status cslbm_state_bytes(const cslbm_ctx* ctx, size_t* bytes);
 cslbm_status cslbm_save_state(cslbm_ctx* ctx, void* buf, size_t bytes, int on_device);
 cslbm_status cslbm_load_state(cslbm_ctx* ctx, const void* buf, size_t bytes, int on_device);
 
+/* One LBM step (cslbm_step) from the saved state `in` to the saved state
+ * `out`, both in the form of cslbm_save_state, with the context's geometry and
+ * boundary velocities; the context's own state stays as it is.  The gather
+ * pass, whatever step_kernel says (the same results up to rounding).  Device
+ * memory of at least cslbm_state_bytes each, not overlapping, aligned to the
+ * storage type (EINVAL otherwise); EINVAL for FP16/BF16 storage.  A caller that
+ * keeps a trajectory spares the copies of save and load.  Asynchronous; both
+ * buffers are in use until the context's stream has run the call. */
+cslbm_status cslbm_step_state(cslbm_ctx* ctx, const void* in, void* out, size_t bytes);
+
 /* Profiling.  While enabled, each LBM step enqueued by cslbm_step is
  * bracketed by CUDA events on the context's stream and every kernel launch
  * of the library is counted.  Enabling resets the counters. */
@@ -266,6 +276,12 @@ cslbm_status cslbm_adjoint_seed_wall_force(cslbm_ctx* ctx, int axis, int side, c
  * from after the step to before it and the step's geometry derivatives are
  * added. */
 cslbm_status cslbm_step_backward(cslbm_ctx* ctx);
+
+/* cslbm_step_backward from a saved state (device memory in the form of
+ * cslbm_save_state) instead of the context's own, which stays as it is.
+ * EINVAL for a buffer that is null, short, misaligned for the storage type or
+ * not device memory. */
+cslbm_status cslbm_step_backward_state(cslbm_ctx* ctx, const void* state, size_t bytes);
 
 /* The adjoint of the rest initialisation (f = f^eq(rho = 1, u = 0), the
  * history F(-1) := F(0)): adds its geometry derivatives. */

@@ -64,12 +64,14 @@ SIGNATURES = {
     "cslbm_state_bytes": [_P, ctypes.POINTER(_SZ)],
     "cslbm_save_state": [_P, _P, _SZ, _I],
     "cslbm_load_state": [_P, _P, _SZ, _I],
+    "cslbm_step_state": [_P, _P, _P, _SZ],
     "cslbm_profile_enable": [_P, _I],
     "cslbm_profile_read": [_P, _D, ctypes.POINTER(ctypes.c_longlong), ctypes.POINTER(ctypes.c_longlong)],
     "cslbm_adjoint_workspace_bytes": [_P, ctypes.POINTER(_SZ)],
     "cslbm_adjoint_attach": [_P, _P, _SZ],
     "cslbm_adjoint_seed_wall_force": [_P, _I, _I, _D],
     "cslbm_step_backward": [_P],
+    "cslbm_step_backward_state": [_P, _P, _SZ],
     "cslbm_adjoint_init_backward": [_P],
     "cslbm_adjoint_metric_grad": [_P, _P, _P, _P, _P, _P],
     "cslbm_transform_interp_scratch_bytes": [_P, ctypes.POINTER(_SZ)],

@@ -91,8 +91,13 @@ class Adjoint:
         e = (ctypes.c_double * 3)(*[float(v) for v in e3])
         call("cslbm_adjoint_seed_wall_force", self.lat.ctx, int(axis), int(side), e)
 
-    def step_backward(self):
-        call("cslbm_step_backward", self.lat.ctx)
+    def step_backward(self, state=None):
+        """The adjoint of the step from the lattice's state, or from a saved one."""
+        if state is None:
+            call("cslbm_step_backward", self.lat.ctx)
+            return
+        call("cslbm_step_backward_state", self.lat.ctx, state.data_ptr(), state.numel())
+        self.lat._hold(state)
 
     def init_backward(self):
         call("cslbm_adjoint_init_backward", self.lat.ctx)
@@ -153,14 +158,14 @@ def _make_function():
             lat.load_state(ctx.final)
             adj.seed_wall_force(ctx.axis, ctx.side, [scale * v for v in ctx.e3])
             for t0, k, ck in reversed(ctx.ckpts):
-                lat.load_state(ck)
-                states = []
-                for _ in range(k):
-                    states.append(lat.save_state())
-                    lat.step(1)
+                # the segment's states, each stepped straight into a buffer of its own
+                states = [ck]
+                for _ in range(k - 1):
+                    states.append(lat.step_state(states[-1]))
                 for st in reversed(states):
-                    lat.load_state(st)
-                    adj.step_backward()
+                    adj.step_backward(st)
+            if ctx.ckpts:
+                lat.load_state(ctx.ckpts[0][2])  # the lattice ends in the state before the first step
             adj.init_backward()
             o6, o18, o9 = adj.metric_grad(g6, dg18)
             return o6, o18, o9, None, None, None, None, None, None

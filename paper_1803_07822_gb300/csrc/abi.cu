@@ -282,6 +282,16 @@ cslbm_status run_metric(cslbm_ctx* c, const double* g6, const double* dg18, int 
 
 cslbm_status cslbm_record_error(cslbm_status s, const char* msg) { return fail(s, msg); }
 
+bool cslbm_is_device_memory(const void* p)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+}
+
 namespace {
 
 // The row-staged step pass: plan and tensor maps, when the storage, shape
@@ -447,16 +457,6 @@ cslbm_status cslbm_set_metric(cslbm_ctx* c, const double* g6, const double* dg18
     return run_metric(c, g6, dg18, on_device, c->gc, true);
 }
 
-static bool is_device_memory(const void* p)
-{
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
-}
-
 cslbm_status cslbm_transform_interp_scratch_bytes(const cslbm_ctx* c, size_t* bytes)
 {
     if (!c || !bytes) return fail(CSLBM_EINVAL, "null argument");
@@ -471,7 +471,7 @@ cslbm_status cslbm_update_metric_interp(cslbm_ctx* c, const double* g6, const do
     if (!c->has_state) return fail(CSLBM_ESTATE, "update_metric_interp before init_equilibrium");
     if (!scratch || scratch_bytes < 20 * (size_t)c->N * c->r_bytes) return fail(CSLBM_ENOMEM, "scratch too small");
     for (const void* q : {(const void*)g6, (const void*)dg18, (const void*)Jnew9, (const void*)psi3, (const void*)scratch})
-        if (!is_device_memory(q)) return fail(CSLBM_EINVAL, "every array of update_metric_interp is device memory");
+        if (!cslbm_is_device_memory(q)) return fail(CSLBM_EINVAL, "every array of update_metric_interp is device memory");
     int* bad = (int*)(c->scratch + 32);
     if (!c->metric_check_pending) CUDA_TRY(cudaMemsetAsync(bad, 0, sizeof(int), c->stream));
     c->ops->transform_interp(c, g6, dg18, Jnew9, psi3, scratch, bad);
@@ -532,7 +532,7 @@ cslbm_status cslbm_update_metric_mixed(cslbm_ctx* c, const double* g6, const flo
     if (!c || !g6 || !dg18 || !Jnew9) return fail(CSLBM_EINVAL, "null argument");
     if (c->r_bytes == 8) return fail(CSLBM_EINVAL, "FP64 storage takes its derivatives and Jacobian in FP64");
     for (const void* q : {(const void*)g6, (const void*)dg18, (const void*)Jnew9})
-        if (!is_device_memory(q)) return fail(CSLBM_EINVAL, "every array of update_metric_mixed is device memory");
+        if (!cslbm_is_device_memory(q)) return fail(CSLBM_EINVAL, "every array of update_metric_mixed is device memory");
     if (!c->has_state) return fail(CSLBM_ESTATE, "update_metric before init_equilibrium");
     int* bad = (int*)(c->scratch + 32);
     if (!c->metric_check_pending) CUDA_TRY(cudaMemsetAsync(bad, 0, sizeof(int), c->stream));
@@ -572,7 +572,7 @@ cslbm_status cslbm_init_equilibrium(cslbm_ctx* c, const double* rho, const doubl
     // forcing of the initial state, F(x, -dt) := F(x, 0)
     c->ops->momentum_field(c);
     LAUNCH_CHECK("momentum kernel");
-    c->ops->step(c, 1);
+    c->ops->step(c, STEP_FORCE_ONLY);
     LAUNCH_CHECK("forcing kernel");
     c->hc ^= 1;
     c->ops->half_shift(c);
@@ -610,7 +610,7 @@ cslbm_status cslbm_step(cslbm_ctx* c, int nsteps)
             c->ev.push_back(e[1]);
             CUDA_TRY(cudaEventRecord(e[0], c->stream));
         }
-        c->launches += c->ops->step(c, 0);
+        c->launches += c->ops->step(c, STEP_ANY);
         LAUNCH_CHECK("step kernel");
         if (c->prof) {
             CUDA_TRY(cudaEventRecord(c->ev.back(), c->stream));
@@ -745,6 +745,24 @@ cslbm_status cslbm_load_state(cslbm_ctx* c, const void* buf, size_t bytes, int o
     CUDA_TRY(cudaMemcpyAsync(c->H[c->hc], (const char*)buf + pb, need - pb, k, c->stream));
     if (!on_device) CUDA_TRY(cudaStreamSynchronize(c->stream));
     c->has_state = 1;
+    return CSLBM_OK;
+}
+
+cslbm_status cslbm_step_state(cslbm_ctx* c, const void* in, void* out, size_t bytes)
+{
+    size_t need = 0;
+    if (cslbm_status s = cslbm_state_bytes(c, &need)) return s;
+    if (c->p.storage != CSLBM_FP32 && c->p.storage != CSLBM_FP64)
+        return fail(CSLBM_EINVAL, "step_state serves FP32 and FP64 storage");
+    if (!in || !out || bytes < need) return fail(CSLBM_EINVAL, "buffer null or too small");
+    const char *a = (const char*)in, *b = (const char*)out;
+    if (((uintptr_t)a | (uintptr_t)b) % c->s_bytes || (a < b + need && b < a + need))
+        return fail(CSLBM_EINVAL, "buffers misaligned or overlapping");
+    if (!cslbm_is_device_memory(in) || !cslbm_is_device_memory(out))
+        return fail(CSLBM_EINVAL, "the states of step_state are device memory");
+    StateSwap swap(c, in, out);
+    c->launches += c->ops->step(c, STEP_GATHER);
+    LAUNCH_CHECK("step kernel");
     return CSLBM_OK;
 }
 

@@ -32,6 +32,7 @@
 // shared memory asynchronously and face nodes run in blocks of their own.
 // 64 x 128 x 64 FP32, us per backward step: A 175 -> 87,
 // the pull of a pass of its own 29 -> 0 (B below).
+#include <cstdint>
 #include <cstdio>
 #include <string>
 
@@ -792,6 +793,17 @@ cslbm_status cslbm_step_backward(cslbm_ctx* c)
     else cslbm::adj::backward<float>(c);
     c->launches += 5;
     return launched("adjoint step");
+}
+
+cslbm_status cslbm_step_backward_state(cslbm_ctx* c, const void* state, size_t bytes)
+{
+    if (cslbm_status s = adj_ready(c)) return s;
+    size_t need = 0;
+    if (cslbm_status s = cslbm_state_bytes(c, &need)) return s;
+    if (!state || bytes < need || (uintptr_t)state % c->s_bytes || !cslbm_is_device_memory(state))
+        return afail(CSLBM_EINVAL, "state null, too small, misaligned or not device memory");
+    StateSwap swap(c, state, nullptr);
+    return cslbm_step_backward(c);
 }
 
 cslbm_status cslbm_adjoint_init_backward(cslbm_ctx* c)

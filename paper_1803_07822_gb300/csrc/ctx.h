@@ -75,6 +75,8 @@ struct cslbm_ctx {
     long long launches;
 };
 
+enum { STEP_ANY = 0, STEP_FORCE_ONLY = 1, STEP_GATHER = 2 };
+
 // Per-storage-format entry points (one kernel unit per format).
 // Node ranges: a launch touches nodes [v0, v0 + cnt); FP64 inputs given as
 // [components][stride] with the node's entry at (v - v0).
@@ -88,9 +90,10 @@ struct cslbm_ops {
     // jf <- rho u of the current state
     void (*momentum_field)(const cslbm_ctx*);
     // one time step P[pc],H[hc] -> P[1-pc],H[1-hc] (momentum pass + step
-    // pass); force_only: only H[1-hc] from the momentum field jf.  Returns
-    // the number of kernels it launched.
-    int (*step)(cslbm_ctx*, int force_only);
+    // pass); FORCE_ONLY: only H[1-hc] from the momentum field jf; GATHER: by
+    // the gather pass whatever applies.  Returns the number of kernels it
+    // launched.
+    int (*step)(cslbm_ctx*, int mode);
     // P[pc] slots -= F/2 of H[hc] (end of initialisation)
     void (*half_shift)(const cslbm_ctx*);
     // chart change for nodes [v0, v0+cnt): P[pc],H[hc],G[gc] -> P[1-pc],H[1-hc] with G[1-gc]
@@ -118,6 +121,35 @@ struct cslbm_ops {
     // acc[0] += number of unstable nodes
     void (*check)(const cslbm_ctx*, double* acc);
 };
+
+// A context whose current state is a saved one for the time of a call: `in`
+// the current populations and history, `out` (or null) the spare ones.
+struct StateSwap {
+    cslbm_ctx* c;
+    void *P0, *P1, *H0, *H1;
+    StateSwap(cslbm_ctx* ctx, const void* in, void* out) : c(ctx), P0(c->P[c->pc]), P1(c->P[1 - c->pc]), H0(c->H[c->hc]), H1(c->H[1 - c->hc])
+    {
+        const size_t pb = 19 * (size_t)c->N * c->s_bytes;
+        c->P[c->pc] = const_cast<void*>(in);
+        c->H[c->hc] = (char*)const_cast<void*>(in) + pb;
+        if (out) {
+            c->P[1 - c->pc] = out;
+            c->H[1 - c->hc] = (char*)out + pb;
+        }
+    }
+    ~StateSwap()
+    {
+        c->P[c->pc] = P0;
+        c->P[1 - c->pc] = P1;
+        c->H[c->hc] = H0;
+        c->H[1 - c->hc] = H1;
+    }
+    StateSwap(const StateSwap&) = delete;
+    StateSwap& operator=(const StateSwap&) = delete;
+};
+
+// device (or managed) memory?
+bool cslbm_is_device_memory(const void* p);
 
 // flag the row-staged step pass sets when one of its bounded waits runs out
 // (an int in the reduction scratch, zero from creation; cslbm_check reads it)

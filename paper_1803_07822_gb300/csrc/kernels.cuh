@@ -1009,13 +1009,17 @@ template <class S, class R> struct Launch {
     {
         launch_momentum<S, R>(c, make_lat(c), P(c, c->pc), H(c, c->hc), G(c, c->gc));
     }
-    static int step(cslbm_ctx* c, int force_only)
+    static int step(cslbm_ctx* c, int mode)
     {
         Lat L = make_lat(c);
-        if (force_only) {
+        if (mode == STEP_FORCE_ONLY) {
             k_forcing<S, R><<<nblocks(c->N), TPB, 0, c->stream>>>(L, P(c, c->pc), H(c, c->hc), H(c, 1 - c->hc),
                                                                  G(c, c->gc), c->jf);
             return 1;
+        }
+        if (mode == STEP_GATHER) {
+            launch_flat_step<S, R>(c, L, P(c, c->pc), P(c, 1 - c->pc), H(c, c->hc), H(c, 1 - c->hc), G(c, c->gc));
+            return 2;
         }
         if constexpr (!std::is_same<R, double>::value) {
             // (a fused launch that the test hook asked for is taken at any size)

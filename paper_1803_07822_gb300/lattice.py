@@ -252,6 +252,14 @@ class CurvedLattice:
     def load_state(self, buf):
         call("cslbm_load_state", self.ctx, buf.data_ptr(), buf.numel(), 1)
 
+    def step_state(self, state):
+        """The saved state one step after the saved state `state` (the
+        lattice's own state stays as it is; FP32 or FP64 storage)."""
+        out = _torch().empty_like(state)
+        call("cslbm_step_state", self.ctx, state.data_ptr(), out.data_ptr(), out.numel())
+        self._hold(state, out)
+        return out
+
     def profile(self, enable=True):
         """Start (or stop) event timing of each LBM step and launch counting."""
         call("cslbm_profile_enable", self.ctx, int(bool(enable)))
