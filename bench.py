@@ -69,10 +69,14 @@ def step_pass(n, storage, step_kernel, axis2_periodic=False):
     rows = (step_kernel in ("auto", "rows") and sb is not None and n[0] <= 256 and n[0] % 4 == 0
             and (n[0] * sb) % 16 == 0 and n[0] * n[1] * n[2] >= 256)
     if rows and step_kernel == "auto":
-        tr = min(256 // n[0], n[1])
-        if tr * n[0] != 256 or n[0] * n[1] * n[2] < (3 << 20 if sb == 4 else 12 << 20):
+        tr, N = min(256 // n[0], n[1]), n[0] * n[1] * n[2]
+        if tr * n[0] != 256 or n[0] < 128:
             return "flat"
-        return "rows" if axis2_periodic else "fused"
+        if axis2_periodic:
+            return "rows" if N >= (1 << 20 if sb == 4 else 2 << 20) else "flat"
+        if sb == 4:
+            return "fused" if N >= 6 << 20 else ("rows" if N >= 2 << 20 else "flat")
+        return "rows" if N >= 6 << 20 else "flat"
     return "rows" if rows else "flat"
 
 

@@ -75,11 +75,14 @@ typedef struct {
  * n[0] <= 256, n[0] a multiple of 4, n[0] * bytes per stored population a
  * multiple of 16 and at least 256 nodes.  Its fused form also forms the
  * momentum field in the same (cooperative) launch; it needs axis 2 to be
- * non-periodic.  AUTO takes the fused row pass, else the row pass, where they
- * apply and pay (256 a multiple of n[0]; at least 3,145,728 nodes in FP32,
- * 12,582,912 in FP16 / BF16), else the flat gather pass; ROWS the row pass
- * (momentum field in a kernel of its own) where it applies, else the flat
- * pass; FLAT always the flat pass.  All give the same results up to rounding. */
+ * non-periodic.  AUTO takes a row pass where one applies and pays, else the
+ * flat gather pass: with n[0] 128 or 256 dividing into tiles of 256 nodes
+ * (n[0] = 128 needs n[1] >= 2), axis 2 periodic: the row pass from 2^20 nodes
+ * in FP32 and 2^21 in FP16 / BF16; else in FP32 the row pass from 2^21 and the
+ * fused one from 6 2^20 nodes, in FP16 / BF16 the row pass from 6 2^20.  ROWS
+ * takes the row pass (momentum field in a kernel of its own) where it
+ * applies, else the flat pass; FLAT always the flat pass.  All give the same
+ * results up to rounding. */
 typedef enum { CSLBM_STEP_AUTO = 0, CSLBM_STEP_FLAT = 1, CSLBM_STEP_ROWS = 2 } cslbm_step_kernel;
 
 typedef struct cslbm_ctx cslbm_ctx;

@@ -301,7 +301,7 @@ void rows_prepare(cslbm_ctx* c)
     cslbm_rows& R = c->rows;
     R.ok = 0;
     R.fused_ok = 0;
-    R.pays = 0;
+    R.best = cslbm::rows::GATHER;
     R.epoch = 0;
     R.test_wait_ns = 0;
     R.test_withhold = -1;
@@ -359,7 +359,7 @@ void rows_prepare(cslbm_ctx* c)
     ok = ok && mk(&R.jf3, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, c->jf, jd3, js3, jb3);
     if (!ok) return;
     R.ok = 1;
-    R.pays = cslbm::rows::pays(R.plan, c->n, (int)c->s_bytes);
+    R.best = cslbm::rows::best_pass(R.plan, c->n, (int)c->s_bytes, c->p.bc_lo[2] == CSLBM_PERIODIC);
     // the fused form: momentum and step in one cooperative launch
     int coop = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device);

@@ -19,7 +19,7 @@ struct cslbm_ops;
 struct cslbm_rows {
     int ok;        // the row pass applies (plan and maps made)
     int fused_ok;  // ... and the fused form (non-periodic axis 2, cooperative launch, smem)
-    int pays;      // AUTO takes them (rows::pays)
+    int best;      // the pass AUTO takes (rows::best_pass)
     cslbm::rows::Plan plan;
     CUtensorMap pop[2];   // [19][n2][n1][n0] populations, box n0 x TR
     CUtensorMap pop3[2];  // the same, box n0 x TR x 1 x 3 (three planes that pull from one row)

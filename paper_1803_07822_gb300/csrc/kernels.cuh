@@ -1024,11 +1024,11 @@ template <class S, class R> struct Launch {
         if constexpr (!std::is_same<R, double>::value) {
             // (a fused launch that the test hook asked for is taken at any size)
             const bool aut = c->p.step_kernel == CSLBM_STEP_AUTO;
-            if (c->rows.fused_ok && aut && (c->rows.pays || c->rows.test_wait_ns)) {
+            if (c->rows.fused_ok && aut && (c->rows.best == rows::FUSED || c->rows.test_wait_ns)) {
                 const int k = launch_fused_step<S>(c, L, c->pc, c->hc, c->gc, step_error_flag(c));
                 if (k > 0) return k;
             }
-            if (c->rows.ok && (!aut || c->rows.pays)) return launch_rows_step<S>(c, L, c->pc, c->hc, c->gc, step_error_flag(c));
+            if (c->rows.ok && (!aut || c->rows.best != rows::GATHER)) return launch_rows_step<S>(c, L, c->pc, c->hc, c->gc, step_error_flag(c));
         }
         launch_flat_step<S, R>(c, L, P(c, c->pc), P(c, 1 - c->pc), H(c, c->hc), H(c, 1 - c->hc), G(c, c->gc));
         return 2;

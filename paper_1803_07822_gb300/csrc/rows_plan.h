@@ -62,17 +62,28 @@ inline bool make_plan(const int n[3], bool yper, bool zper, int s_bytes, int max
     return (long long)smem_bytes(pl) <= max_smem;
 }
 
-// Whether the row passes beat the gather pass where they apply.  They need
-// full tiles (TR n0 = NT: all compute threads busy, grouped copies; 192-node
-// rows: 742 us fused, 574 gather at 192^3 FP32) and a lattice well beyond L2,
-// where one read of the populations less counts: measured in us per step,
-// fused / gather, FP32 128^3 192 / 175, 256x256x48 264 / 271, 256x256x96
-// 463 / 515, 256^3 1,138 / 1,334; FP16 256x256x96 444 / 431, 256x256x192
-// 818 / 838.  Hence 3.1 million nodes for FP32, 12.6 million for 16 bits.
-inline bool pays(const Plan& pl, const int n[3], int s_bytes)
+// The pass AUTO takes where the row passes apply.  They need full tiles (TR n0 =
+// NT: all compute threads busy, grouped copies; 192-node rows: 742 us fused,
+// 574 gather at 192^3 FP32) of one or two rows (four rows of 64: 103 rows, 87
+// gather at 64x128x128) and enough nodes to fill the copy pipeline; the
+// fused form pays its waits back only well beyond L2.  us per step:
+//   FP32, walls across axis 2    gather  rows  fused   | periodic  gather  rows
+//     256x256x16   (1.0 M)         93     95    112    |             86     78
+//     256x256x32   (2.1 M)        174    168    181    |            167    153
+//     128x256x128  (4.2 M)        333    316    322    |            329    304
+//     256x256x128  (8.4 M)        660    595    571    |            652    578
+//   16 bits
+//     256x256x32                  148    153    171    |            139    135
+//     256x256x48   (3.1 M)        217    216    234    |            208    199
+//     256x256x128                 553    529    546    |            543    513
+enum Pass { GATHER = 0, ROWS = 1, FUSED = 2 };
+inline Pass best_pass(const Plan& pl, const int n[3], int s_bytes, bool zper)
 {
     const long long N = (long long)n[0] * n[1] * n[2];
-    return pl.TR * n[0] == NT && N >= (s_bytes == 4 ? 3LL << 20 : 12LL << 20);
+    if (pl.TR * n[0] != NT || n[0] < 128) return GATHER;
+    if (zper) return N >= (s_bytes == 4 ? 1LL << 20 : 2LL << 20) ? ROWS : GATHER;
+    if (s_bytes == 4) return N >= 6LL << 20 ? FUSED : (N >= 2LL << 20 ? ROWS : GATHER);
+    return N >= 6LL << 20 ? ROWS : GATHER;
 }
 
 // smem layout of the fused pass after the two step stages: the momentum
