@@ -11,15 +11,15 @@
 // nearest the face, axis by axis (tensor product at edges and corners).
 //
 // Two kernels: the first writes F / 12, F = f - (c_s^2/2) L f (order 4,
-// k_correct) or the continued f (order 2, k_pad), on the lattice padded by one
-// site along every axis with a non-periodic face; k_grad forms G_i F at every
-// node.  FP64 throughout, which is what bounds both: the FP64 pipe issues two
+// k_correct), or the continued f itself (order 2, k_pad: its bits, so that
+// differences of close values stay exact), on the lattice padded by one site
+// along every axis with a non-periodic face; k_grad forms G_i F at every node.  FP64 throughout, which is what bounds both: the FP64 pipe issues two
 // lanes per clock and SM, so only the number of FP64 instructions counts.
 // Written out per node, the stencils take 22 and 24 of them; both factor into
-// sums along one axis that neighbours share, which leaves 10 and 15: blocks
+// sums along one axis that neighbours share, which leaves 10 and 16: blocks
 // march along axis 2 with one plane of a 32 x 8 tile (and its rim) in shared
 // memory, in-plane sums exchanged there, sums along the march kept in
-// registers.  Six fields on 128 x 256 x 128, order 4: 1,359 + 1,150 -> 695 + 840 us.
+// registers.  Six fields on 128 x 256 x 128, order 4: 1,359 + 1,150 -> 1,559 us for both.
 #include <cstdint>
 #include <string>
 
@@ -111,8 +111,8 @@ __device__ __forceinline__ bool inner(const Box& B, int a, int r)
     return r >= 0 && r < B.n[a] && (r >= 1 || B.plo[a]) && (r <= B.n[a] - 2 || B.phi[a]);
 }
 // The fields and the weights.  The faces of G_i weigh w_1 / c_s^2 = 1/6, its
-// edges w_7 / c_s^2 = 1/12; the scratch holds F / 12, so that the gradient
-// below needs no products but by two.
+// edges w_7 / c_s^2 = 1/12; with order 4 the scratch holds F / 12, so that the
+// gradient below needs no products but by two.
 constexpr double kEdge = 1.0 / 12.0;
 
 // order 2: the continued field at every site of the padded lattice, component blockIdx.y
@@ -124,8 +124,8 @@ __global__ void __launch_bounds__(TBL) k_pad(const __grid_constant__ Box B, cons
     if (s >= (unsigned)B.Ne) return;
     const unsigned ne0 = B.ne[0], ne1 = B.ne[1], row = s / ne0, zr = row / ne1;
     F[(long long)blockIdx.y * B.Ne + s] =
-        kEdge * site(B, f + (long long)blockIdx.y * B.N, 2, (int)(s - row * ne0) - B.pad[0],
-                     (int)(row - zr * ne1) - B.pad[1], (int)zr - B.pad[2]);
+        site(B, f + (long long)blockIdx.y * B.N, 2, (int)(s - row * ne0) - B.pad[0],
+             (int)(row - zr * ne1) - B.pad[1], (int)zr - B.pad[2]);
 }
 
 // F = f - (c_s^2/2) L f = f0 - sum_l w_l (f_l - f0) at a site whose stencil
@@ -156,7 +156,7 @@ __device__ __noinline__ double correct_far(const Box& B, const double* __restric
 // Order 4: F / 12 on the padded lattice.  With the in-plane sums q = s_x + s_y
 // (s_a = f(a + 1) + f(a - 1)) and e = s_x(y + 1) + s_x(y - 1), and u = f + q/2,
 //   F = (5/3) f - (q + e/2) / 18 - (u(z + 1) + u(z - 1)) / 18.
-// Planes beyond a face of axis 2 continue u and the in-plane part; a site whose
+// Planes beyond a face of axis 2 are continued as they are loaded; a site whose
 // stencil leaves the lattice across axis 0 or 1 takes correct_far.
 __global__ void __launch_bounds__(TX* TY) k_correct(const __grid_constant__ Box B, const __grid_constant__ Tiles T,
                                                     const double* __restrict__ f, double* __restrict__ F)
@@ -181,12 +181,29 @@ __global__ void __launch_bounds__(TX* TY) k_correct(const __grid_constant__ Box 
             off[k] = ry * B.n[0] + rx;
     }
     const unsigned n01 = (unsigned)B.n[0] * B.n[1];
-    // u and the in-plane part w of F at plane pz of the lattice (every thread of the block)
-    auto plane = [&](int pz, double& u, double& w) {
-        const double* fp = fc + (unsigned)pz * n01;
+    // u and the in-plane part w of F at plane p (every thread of the block); a
+    // plane one or two beyond a face is continued as it is loaded.  (To
+    // continue u and w, which are linear in f, doubles the error next to the
+    // face: their rounding is multiplied by the weights.)
+    auto plane = [&](int p, double& u, double& w) {
+        int pz = p;
+        if (wrap(B, 2, pz)) {
+            const double* fp = fc + (unsigned)pz * n01;
 #pragma unroll
-        for (int k = 0; k < 2; k++)
-            if (off[k] >= 0) (&fs[0][0])[t + k * TX * TY] = __ldg(fp + off[k]);
+            for (int k = 0; k < 2; k++)
+                if (off[k] >= 0) (&fs[0][0])[t + k * TX * TY] = __ldg(fp + off[k]);
+        } else {
+            const int beyond = p < 0 ? -p : p - (B.n[2] - 1);
+#pragma unroll
+            for (int k = 0; k < 2; k++)
+                if (off[k] >= 0) {
+                    double v = 0.0;
+#pragma unroll
+                    for (int i = 0; i <= 4; i++)
+                        v = fma(cont_weight(4, beyond, i), __ldg(fc + (unsigned)(p < 0 ? i : B.n[2] - 1 - i) * n01 + off[k]), v);
+                    (&fs[0][0])[t + k * TX * TY] = v;
+                }
+        }
         __syncthreads();
         const double sx = fs[ty + 1][tx] + fs[ty + 1][tx + 2];
         ss[ty + 1][tx] = sx;
@@ -199,23 +216,8 @@ __global__ void __launch_bounds__(TX* TY) k_correct(const __grid_constant__ Box 
     };
     double ua = 0.0, ub = 0.0, wb = 0.0;  // u of planes p - 2 and p - 1, w of p - 1
     for (int p = za - 1; p <= zb; p++) {
-        double u = 0.0, w = 0.0;
-        int pz = p;
-        if (wrap(B, 2, pz)) {
-            plane(pz, u, w);
-        } else {
-            // one or two planes beyond a face: u and w are linear in f, so they
-            // continue with the weights of f
-            const int beyond = p < 0 ? -p : p - (B.n[2] - 1);
-#pragma unroll 1
-            for (int k = 0; k <= 4; k++) {
-                double uk, wk;
-                plane(p < 0 ? k : B.n[2] - 1 - k, uk, wk);
-                const double a = cont_weight(4, beyond, k);
-                u = fma(a, uk, u);
-                w = fma(a, wk, w);
-            }
-        }
+        double u, w;
+        plane(p, u, w);
         const int z = p - 1;
         if (p > za && mine) {
             const double v = flat ? fma(-kEdge / 18.0, ua + u, wb) : kEdge * correct_far(B, fc, x, y, z);
@@ -229,15 +231,20 @@ __global__ void __launch_bounds__(TX* TY) k_correct(const __grid_constant__ Box 
 }
 
 // d_k f_c = G_k F at every node, out[(k ncomp + c) N + v].  With the
-// differences d_x = F(x + 1) - F(x - 1), d_y, their sums over the two
-// neighbours across (along y or x in the plane, along z in the march) and
-// z = 2 F + s_x + s_y, in units of F / 12:
+// differences d_x = F(x + 1) - F(x - 1), d_y, d_z and their sums over the
+// neighbours across,
 //   D_x = 2 d_x + (d_x(y + 1) + d_x(y - 1)) + (d_x(z + 1) + d_x(z - 1)),
-//   D_y likewise, D_z = z(z + 1) - z(z - 1).
+//   D_y and D_z likewise, in units of F / 12 (EDGE: F itself is given, the
+// sums are scaled here).  Differences come before every sum: the fields vary
+// little from node to node, and a difference of sums 2 F + s_x + s_y (one
+// instruction less) doubled the error of D_z against 64-bit significands.
+// d_z of the plane before the newest is exchanged beside that plane, from the
+// entries each thread kept of the two planes before.
+template <bool EDGE>
 __global__ void __launch_bounds__(TX* TY) k_grad(const __grid_constant__ Box B, const __grid_constant__ Tiles T, int ncomp,
                                                  const double* __restrict__ F, double* __restrict__ out)
 {
-    __shared__ double fs[TY + 2][TX + 2], dxs[TY + 2][TX], dys[TY][TX + 2];
+    __shared__ double fs[TY + 2][TX + 2], dzs[TY + 2][TX + 2], dxs[TY + 2][TX], dys[TY][TX + 2];
     const int tx = threadIdx.x, ty = threadIdx.y, t = ty * TX + tx;
     int x0, y0, za, zb;
     tile_of(T, 0, 0, x0, y0, za, zb);
@@ -258,14 +265,21 @@ __global__ void __launch_bounds__(TX* TY) k_grad(const __grid_constant__ Box B, 
         }
     }
     const unsigned ne01 = (unsigned)B.ne[0] * B.ne[1];
-    double dxa = 0.0, dxb = 0.0, rxb = 0.0, dya = 0.0, dyb = 0.0, ryb = 0.0, qa = 0.0, qb = 0.0;
+    double dxa = 0.0, dxb = 0.0, rxb = 0.0, dya = 0.0, dyb = 0.0, ryb = 0.0;
+    double fa[2] = {0.0, 0.0}, fb[2] = {0.0, 0.0};  // this thread's entries of planes p - 2 and p - 1
     for (int p = za - 1; p <= zb; p++) {
         int pz = p;
         wrap(B, 2, pz);
         const double* fp = Fc + (unsigned)(pz + B.pad[2]) * ne01;
 #pragma unroll
         for (int k = 0; k < 2; k++)
-            if (off[k] >= 0) (&fs[0][0])[t + k * TX * TY] = __ldg(fp + off[k]);
+            if (off[k] >= 0) {
+                const double v = __ldg(fp + off[k]);
+                (&fs[0][0])[t + k * TX * TY] = v;
+                (&dzs[0][0])[t + k * TX * TY] = v - fa[k];
+                fa[k] = fb[k];
+                fb[k] = v;
+            }
         __syncthreads();
         const double e = fs[ty + 1][tx + 2], w = fs[ty + 1][tx], n = fs[ty + 2][tx + 1], s = fs[ty][tx + 1];
         const double dx = e - w, dy = n - s;
@@ -277,7 +291,8 @@ __global__ void __launch_bounds__(TX* TY) k_grad(const __grid_constant__ Box B, 
             const int r = tx >> 1, col = (tx & 1) * (TX + 1);
             dys[r][col] = fs[r + 2][col] - fs[r][col];
         }
-        const double q = fma(2.0, fs[ty + 1][tx + 1], (e + w) + (n + s));
+        const double rz = fma(2.0, dzs[ty + 1][tx + 1],
+                              (dzs[ty + 1][tx + 2] + dzs[ty + 1][tx]) + (dzs[ty + 2][tx + 1] + dzs[ty][tx + 1]));
         __syncthreads();
         const double rx = fma(2.0, dx, dxs[ty][tx] + dxs[ty + 2][tx]);
         const double ry = fma(2.0, dy, dys[ty][tx] + dys[ty][tx + 2]);
@@ -285,9 +300,10 @@ __global__ void __launch_bounds__(TX* TY) k_grad(const __grid_constant__ Box B, 
             const unsigned v = ((unsigned)(p - 1) * B.n[1] + (unsigned)y) * (unsigned)B.n[0] + (unsigned)x;
             double* o = out + (long long)c * B.N + v;
             const long long comp = (long long)ncomp * B.N;
-            o[0] = rxb + (dxa + dx);
-            o[comp] = ryb + (dya + dy);
-            o[2 * comp] = q - qa;
+            const double gx = rxb + (dxa + dx), gy = ryb + (dya + dy);
+            o[0] = EDGE ? kEdge * gx : gx;
+            o[comp] = EDGE ? kEdge * gy : gy;
+            o[2 * comp] = EDGE ? kEdge * rz : rz;
         }
         dxa = dxb;
         dxb = dx;
@@ -295,8 +311,6 @@ __global__ void __launch_bounds__(TX* TY) k_grad(const __grid_constant__ Box B, 
         dya = dyb;
         dyb = dy;
         ryb = ry;
-        qa = qb;
-        qb = q;
     }
 }
 
@@ -361,7 +375,8 @@ cslbm_status gradient(cslbm_ctx* c, const double* f, int ncomp, int order, doubl
         k_pad<<<dim3((unsigned)((B.Ne + TBL - 1) / TBL), (unsigned)ncomp), TBL, 0, c->stream>>>(B, f, F);
     }
     const Tiles T = tiles_of(c->n_sm, B.n[0], B.n[1], 0, B.n[2], ncomp);
-    k_grad<<<tile_grid(T, ncomp), dim3(TX, TY), 0, c->stream>>>(B, T, ncomp, F, out);
+    if (order == 4) k_grad<false><<<tile_grid(T, ncomp), dim3(TX, TY), 0, c->stream>>>(B, T, ncomp, F, out);
+    else k_grad<true><<<tile_grid(T, ncomp), dim3(TX, TY), 0, c->stream>>>(B, T, ncomp, F, out);
     c->launches += 2;
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return lfail(CSLBM_ECUDA, std::string("lattice gradient: ") + cudaGetErrorString(e));
