@@ -398,8 +398,8 @@ def bench_batch(args):
         "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
         "dtype": "f32", "data": "synthetic",
         "config": {"workload": "64 independent deformed periodic channels, sides U{32..96}, 4 modes 2-10 %, "
-                               "tau U[0.55, 1.0], FP32, batched (one persistent launch per LBM step over a "
-                               "work-item queue, CUDA graph)", "nodes": N, "lbm_steps_per_step": STEPS_PER_CYCLE,
+                               "tau U[0.55, 1.0], FP32, batched (one persistent launch per LBM step over "
+                               "work items, CUDA graph)", "nodes": N, "lbm_steps_per_step": STEPS_PER_CYCLE,
                    "l2": "inputs > L2 (5.8 GB of state per LBM step), no flush",
                    "tile_shape": {"block_nodes": shape[0], "item_nodes": shape[1], "blocks_per_sm": shape[2]},
                    "tune_ms_per_lbm_step": {f"{k[0]}/{k[1]}/{k[2]}": v for k, v in sorted(tune_table.items())},
@@ -534,7 +534,7 @@ def bench_d2q9(args):
                        "nodes": N, "lbm_steps_per_step": STEPS_PER_CYCLE,
                        "l2": "inputs > L2 (0.7 GB of state per LBM step), no flush"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                         "traffic": None, "peak_kind": peak_kind, "kernel": "one LBM step: k2_momentum + k2_step",
+                         "traffic": None, "peak_kind": peak_kind, "kernel": "one LBM step: k2_step_march",
                          "bytes_per_node": BYTES_PER_NODE_2D, "step_ms": step_ms},
             "gpu_launches": 2 * STEPS_PER_CYCLE * args.steps, "clocks": clk}
     if not args.no_cpu_baseline:
@@ -629,9 +629,10 @@ def adjoint_report(step_kernel, steps=None):
 
 
 # FP64 operations (an FMA counts 2) per lattice site and field of the
-# lattice-derivative kernels as written: k_pad 16 additions + 2 FMAs + 1
-# multiply per padded site (order 4), k_grad 9 pair differences + 15 FMAs
-LAP_FLOP, GRAD_FLOP = {2: 0, 4: 21}, {2: 39, 4: 39}
+# lattice-derivative kernels as written, rims and overlapping planes of the
+# tiles apart: k_correct 5 additions + 1 multiply + 4 FMAs per padded site
+# (order 4), k_pad 1 multiply (order 2), k_grad 12 additions + 3 FMAs
+LAP_FLOP, GRAD_FLOP = {2: 1, 4: 14}, {2: 18, 4: 18}
 # FP64 peak from the unit counts: 152 SMs x 2 FP64 FMA per clock x 2 x 2.07 GHz
 FP64_PEAK_GFLOPS = 152 * 2 * 2 * 2.07
 
@@ -663,7 +664,7 @@ def lattice_gradient_report(lat, g6, order=4, reps=5):
 
 
 def transform_interp_report(lat, dev, layout, reps=5):
-    """Device time of one chart change of the bench channel (metric kernel +
+    """Device time of one chart change of the bench channel (metric and
     transformation) with the interpolating form against the node-wise one.
     The transition map of the channel chart h^w = x_w (1 + d/H) between two
     snapshots: x_w = x~_w J~^w_w / J^w_w (J^w_w = 1 + d/H), the rest fixed."""
@@ -695,7 +696,7 @@ def transform_interp_report(lat, dev, layout, reps=5):
         torch.cuda.synchronize()
         out[mode] = e0.elapsed_time(e1) / (reps * len(pairs))
     return {"node_wise_ms": out["node"], "interp_ms": out["interp"], "nodes": lat.N,
-            "note": "one chart change incl. the metric kernel; the interpolating form adds the moment-field pass "
+            "note": "one chart change incl. the metric; the interpolating form adds the moment-field pass "
                     "and reads 8 corners per node (20 fields + the Jacobian)"}
 
 

@@ -456,7 +456,7 @@ cslbm_status cslbm2d_set_boundary_velocity(cslbm2d_ctx* ctx, int axis, int side,
  * before the metric is set */
 cslbm_status cslbm2d_init_equilibrium(cslbm2d_ctx* ctx, const double* rho, const double* u2, int on_device);
 /* nsteps LBM steps (Sec. II, Eqs. collision and streaming, with the forcing
- * of Eqs. forcing-A/B/C), two kernels each, asynchronous; ESTATE before
+ * of Eqs. forcing-A/B/C), one kernel each, asynchronous; ESTATE before
  * init_equilibrium */
 cslbm_status cslbm2d_step(cslbm2d_ctx* ctx, int nsteps);
 /* rho [N], u2 [2][N] (Sec. II, Eqs. fields: contravariant, or Cartesian

@@ -304,8 +304,8 @@ def _params(n, bc_lo, bc_hi, tau, theta, fext, storage, literal_a2, step_kernel)
 
 
 class CurvedBatch:
-    """Independent FP32 channels of any sizes advanced together (two kernel
-    launches per step for the whole batch, replayed from a CUDA graph).
+    """Independent FP32 channels of any sizes advanced together (one
+    persistent launch per step for the whole batch, replayed from a CUDA graph).
 
     channels: list of dicts with keys n, bc_lo, bc_hi, tau and optionally
     fext, theta.  batch[i] is a CurvedLattice view of channel i (geometry,
