@@ -81,7 +81,7 @@ def step_pass(n, storage, step_kernel, axis2_periodic=False):
 
 
 PASS_KERNELS = {"fused": "k_step_fused + k_step_faces", "rows": "k_momentum_flat + k_step_rows + k_step_faces",
-                "flat": "k_momentum_flat + k_step_flat"}
+                "flat": "k_momentum_flat (k_momentum_rule where the boundary rule gives rho u of face nodes) + k_step_flat"}
 
 
 def workload_spec(name):

@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(TB, 512 / TB) k_batch_persistent(const Chan* _
         for (unsigned v = v0 + threadIdx.x; v < v1; v += TB) {
             int x, y, z;
             flat_coords(C.L, C.pl, v, x, y, z);
-            momentum_node<float, float>(C.L, C.P[pi], C.H[hi], C.G, C.jf, x, y, z, v);
+            momentum_node<float, float, true>(C.L, C.P[pi], C.H[hi], C.G, C.jf, x, y, z, v);
         }
     }
     grid_barrier(q, err);

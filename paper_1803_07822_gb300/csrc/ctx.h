@@ -87,7 +87,7 @@ struct cslbm_ops {
     // P[pc] slots of f^eq(rho,u) (history still zero)
     void (*init_scatter)(const cslbm_ctx*, const double* rho, const double* u3, long long stride,
                          long long v0, long long cnt);
-    // jf <- rho u of the current state
+    // jf <- rho u of the current state (FP32 arithmetic: of face nodes from the boundary rule)
     void (*momentum_field)(const cslbm_ctx*);
     // one time step P[pc],H[hc] -> P[1-pc],H[1-hc] (momentum pass + step
     // pass); FORCE_ONLY: only H[1-hc] from the momentum field jf; GATHER: by

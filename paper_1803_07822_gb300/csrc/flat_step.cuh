@@ -26,6 +26,7 @@
 #pragma once
 
 #include <mutex>
+#include <type_traits>
 
 #include "fast_div.h"
 #include "step_math.cuh"
@@ -58,21 +59,21 @@ __device__ __forceinline__ unsigned nbr_off(const Nbr& p, int cx, int cy, int cz
     return p.zs[cz + 1] + p.ys[cy + 1] + p.xs[cx + 1];
 }
 
-// rho u of one node into jf[v].  A face node's follows from its inner node
-// without the boundary rule's populations: a wall or inflow node takes
-// rho_i u_w (the first moment of f^eq(rho_i, u_w) plus that of the inner
-// node's non-equilibrium part, which vanishes), an outflow node takes j_i.
-// So every node makes the same gather, a face node at its inner node.
-template <class S, class R>
+// rho u of a node into jf[v].  With FACES every node, a face node's from its
+// inner node without the boundary rule's populations: a wall or inflow node
+// takes rho_i u_w (the first moment of f^eq(rho_i, u_w) plus that of the inner
+// node's non-equilibrium part, which vanishes), an outflow node takes j_i.  So
+// every node makes the same gather, a face node at its inner node.  Without,
+// nodes on no face only.
+template <class S, class R, bool FACES>
 __device__ __forceinline__ void momentum_node(const Lat& L, const S* __restrict__ P, const R* __restrict__ hist,
                                               const R* __restrict__ geo, Mom4<R>* __restrict__ jf, int x, int y,
                                               int z, unsigned v)
 {
     const unsigned N = (unsigned)L.N;
-    const bool face = on_boundary(L, x, y, z);
     const int r[3] = {x, y, z};
     int in[3] = {x, y, z}, axis = 0, side = 0, bc = BC_OUTFLOW;
-    if (face) bc = classify(L, r, axis, side, in);
+    if (FACES && on_boundary(L, x, y, z)) bc = classify(L, r, axis, side, in);
     const Nbr src = nbr_index(L, in[0], in[1], in[2], -1);
     R s[Q];
 #pragma unroll
@@ -92,7 +93,7 @@ __device__ __forceinline__ void momentum_node(const Lat& L, const S* __restrict_
     j.x = fmad(sg, m1[0], R(0.5) * j.x);
     j.y = fmad(sg, m1[1], R(0.5) * j.y);
     j.z = fmad(sg, m1[2], R(0.5) * j.z);
-    if (bc != BC_OUTFLOW) {
+    if (FACES && bc != BC_OUTFLOW) {
         R m0 = s[0];
 #pragma unroll
         for (int k = 0; k < 9; k++) m0 += Ps.p[k];
@@ -103,6 +104,27 @@ __device__ __forceinline__ void momentum_node(const Lat& L, const S* __restrict_
         j.y = rho * u[1];
         j.z = rho * u[2];
     }
+    jf[v] = j;
+}
+
+// rho u of a face node as the first moment of the boundary rule's populations
+template <class S, class R>
+__device__ __noinline__ void momentum_boundary(const Lat& L, const S* __restrict__ P, const R* __restrict__ hist,
+                                               const R* __restrict__ geo, int x, int y, int z, Mom4<R>* jf)
+{
+    R s[Q];
+    boundary_pops<S, R>(L, P, hist, geo, x, y, z, s);
+    PairSums<R> Ps;
+    pair_sums(s, Ps);
+    R m1[3];
+    first_moment(Ps, m1);
+    const long long v = nidx(L, x, y, z);
+    const R sg = geo[v];
+    Mom4<R> j;
+    j.x = fmad(sg, m1[0], R(0.5) * hist[1 * L.N + v]);
+    j.y = fmad(sg, m1[1], R(0.5) * hist[2 * L.N + v]);
+    j.z = fmad(sg, m1[2], R(0.5) * hist[3 * L.N + v]);
+    j.w = R(0);
     jf[v] = j;
 }
 
@@ -138,7 +160,105 @@ __global__ void __launch_bounds__(FB) k_momentum_flat(const __grid_constant__ La
     wait_previous();
     launch_next();
     if (v >= (unsigned)L.N) return;
-    momentum_node<S, R>(L, P, hist, geo, jf, x, y, z, v);
+    momentum_node<S, R, true>(L, P, hist, geo, jf, x, y, z, v);
+}
+
+// The nodes on non-periodic faces as up to six boxes without overlap: the
+// faces of axis 2 whole, those of axis 1 without the axis-2 face nodes, those
+// of axis 0 without the face nodes of axes 1 and 2.
+struct FaceList {
+    int nseg;
+    int lo[6][3], len[6][3];
+    long long start[7];
+};
+
+inline FaceList face_list(const cslbm_ctx* c)
+{
+    FaceList f{};
+    long long total = 0;
+    bool done[3] = {false, false, false};
+    for (int a = 2; a >= 0; a--) {
+        if (c->p.bc_lo[a] == CSLBM_PERIODIC) continue;
+        for (int side = 0; side < 2; side++) {
+            const int k = f.nseg++;
+            for (int b = 0; b < 3; b++) {
+                if (b == a) {
+                    f.lo[k][b] = side ? c->n[b] - 1 : 0;
+                    f.len[k][b] = 1;
+                } else if (done[b]) {
+                    f.lo[k][b] = 1;
+                    f.len[k][b] = c->n[b] - 2;
+                } else {
+                    f.lo[k][b] = 0;
+                    f.len[k][b] = c->n[b];
+                }
+            }
+            f.start[k] = total;
+            total += (long long)f.len[k][0] * f.len[k][1] * f.len[k][2];
+        }
+        done[a] = true;
+    }
+    f.start[f.nseg] = total;
+    return f;
+}
+
+// nodes on non-periodic faces
+inline long long face_count(const cslbm_params& p)
+{
+    long long all = 1, inner = 1;
+    for (int a = 0; a < 3; a++) {
+        all *= p.n[a];
+        inner *= p.bc_lo[a] == CSLBM_PERIODIC ? p.n[a] : p.n[a] - 2;
+    }
+    return all - inner;
+}
+
+// node i of the list; false past its end.  (Selects over the six segments: an
+// index of f by a runtime value would copy it to local memory; face nodes
+// number fewer than 2^31.)
+__device__ __forceinline__ bool face_coords(const FaceList& f, int i, int& x, int& y, int& z)
+{
+    if (i >= (int)f.start[f.nseg]) return false;
+    int lo0 = 0, lo1 = 0, lo2 = 0, len0 = 1, len1 = 1, st = 0;
+#pragma unroll
+    for (int k = 0; k < 6; k++)
+        if (k < f.nseg && i >= (int)f.start[k]) {
+            lo0 = f.lo[k][0];
+            lo1 = f.lo[k][1];
+            lo2 = f.lo[k][2];
+            len0 = f.len[k][0];
+            len1 = f.len[k][1];
+            st = (int)f.start[k];
+        }
+    const int r = i - st, q = r / len0;
+    x = lo0 + (r - q * len0);
+    y = lo1 + q % len1;
+    z = lo2 + q / len1;
+    return true;
+}
+
+// The same with the boundary rule on face nodes (momentum_by_rule), which the
+// first nfb blocks take: 91 x 77 x 93 FP32, ten steps and the fields, 654 -> 659 us
+template <class S, class R>
+__global__ void __launch_bounds__(FB)
+    k_momentum_rule(const __grid_constant__ Lat L, const __grid_constant__ Plane pl, const __grid_constant__ FaceList f,
+                    unsigned nfb, const S* __restrict__ P, const R* __restrict__ hist, const R* __restrict__ geo,
+                    Mom4<R>* __restrict__ jf)
+{
+    int x, y, z;
+    if (blockIdx.x < nfb) {
+        const bool ok = face_coords(f, (int)(blockIdx.x * blockDim.x + threadIdx.x), x, y, z);
+        wait_previous();
+        launch_next();
+        if (ok) momentum_boundary<S, R>(L, P, hist, geo, x, y, z, jf);
+        return;
+    }
+    const unsigned v = (blockIdx.x - nfb) * blockDim.x + threadIdx.x;
+    flat_coords(L, pl, v, x, y, z);
+    wait_previous();
+    launch_next();
+    if (v >= (unsigned)L.N || on_boundary(L, x, y, z)) return;
+    momentum_node<S, R, false>(L, P, hist, geo, jf, x, y, z, v);
 }
 
 // rho u at a stencil site that may lie one step outside a non-periodic face:
@@ -241,11 +361,10 @@ __device__ __forceinline__ void ghost_differences(const Lat& L, const Mom4<R>* j
 #pragma unroll
     for (int k = 0; k < 9; k++) {
         const int l = 2 * k + 1;
-        R acc[3] = {R(0), R(0), R(0)};
+        R site[2][3];  // rho u at x + c_l and at x - c_l, each summed in mom_site's order
 #pragma unroll
-        for (int s = 1; s >= -1; s -= 2) {
-            const int c[3] = {s * cvec(l, 0), s * cvec(l, 1), s * cvec(l, 2)};
-            const R sg = R(s);
+        for (int s = 0; s < 2; s++) {
+            const int sg = 1 - 2 * s, c[3] = {sg * cvec(l, 0), sg * cvec(l, 1), sg * cvec(l, 2)};
             // the (one or two) displaced axes a, b; the others contribute their own coordinate
             const int a = c[0] ? 0 : (c[1] ? 1 : 2), b = c[2] ? 2 : (c[1] ? 1 : 0);
             unsigned rest = 0;
@@ -256,16 +375,15 @@ __device__ __forceinline__ void ghost_differences(const Lat& L, const Mom4<R>* j
             const bool ta = two[a][ia], tb = a != b && two[b][ib];
             const unsigned o0 = rest + o[a][ia], ob = a != b ? o[b][ib] : 0u, gb = a != b ? g[b][ib] : 0u;
             const R wa = ta ? R(2) : R(1), wb = tb ? R(2) : R(1);
-            add(acc, true, sg * wa * wb, o0 + ob);
-            add(acc, ta, -sg * wb, rest + g[a][ia] + ob);
-            if (a != b) {
-                add(acc, tb, -sg * wa, o0 + gb);
-                add(acc, ta && tb, sg, rest + g[a][ia] + gb);
-            }
+            R(&acc)[3] = site[s];
+            acc[0] = acc[1] = acc[2] = R(0);
+            add(acc, true, wa * wb, o0 + ob);
+            if (a != b) add(acc, tb, -wa, o0 + gb);
+            add(acc, ta, -wb, rest + g[a][ia] + ob);
+            if (a != b) add(acc, ta && tb, R(1), rest + g[a][ia] + gb);
         }
-        d[k][0] = acc[0];
-        d[k][1] = acc[1];
-        d[k][2] = acc[2];
+#pragma unroll
+        for (int i = 0; i < 3; i++) d[k][i] = site[0][i] - site[1][i];
     }
 }
 
@@ -398,56 +516,6 @@ __device__ __forceinline__ void step_boundary_body(const Lat& L, const S* __rest
     step_core<S, R>(L, s, G, Hp, d, Pout, hout, v, N);
 }
 
-// The nodes on non-periodic faces as up to six boxes without overlap: the
-// faces of axis 2 whole, those of axis 1 without the axis-2 face nodes, those
-// of axis 0 without the face nodes of axes 1 and 2.
-struct FaceList {
-    int nseg;
-    int lo[6][3], len[6][3];
-    long long start[7];
-};
-
-inline FaceList face_list(const cslbm_ctx* c)
-{
-    FaceList f{};
-    long long total = 0;
-    bool done[3] = {false, false, false};
-    for (int a = 2; a >= 0; a--) {
-        if (c->p.bc_lo[a] == CSLBM_PERIODIC) continue;
-        for (int side = 0; side < 2; side++) {
-            const int k = f.nseg++;
-            for (int b = 0; b < 3; b++) {
-                if (b == a) {
-                    f.lo[k][b] = side ? c->n[b] - 1 : 0;
-                    f.len[k][b] = 1;
-                } else if (done[b]) {
-                    f.lo[k][b] = 1;
-                    f.len[k][b] = c->n[b] - 2;
-                } else {
-                    f.lo[k][b] = 0;
-                    f.len[k][b] = c->n[b];
-                }
-            }
-            f.start[k] = total;
-            total += (long long)f.len[k][0] * f.len[k][1] * f.len[k][2];
-        }
-        done[a] = true;
-    }
-    f.start[f.nseg] = total;
-    return f;
-}
-
-// nodes on non-periodic faces
-inline long long face_count(const cslbm_params& p)
-{
-    long long all = 1, inner = 1;
-    for (int a = 0; a < 3; a++) {
-        all *= p.n[a];
-        inner *= p.bc_lo[a] == CSLBM_PERIODIC ? p.n[a] : p.n[a] - 2;
-    }
-    return all - inner;
-}
-
 // the same out of line, where one kernel runs face nodes among others (jf may
 // be written by the same launch: plain loads)
 template <class S, class R>
@@ -456,30 +524,6 @@ __device__ __noinline__ void step_face(const Lat& L, const S* __restrict__ Pin, 
                                        const Mom4<R>* jf, int x, int y, int z)
 {
     step_boundary_body<S, R>(L, Pin, Pout, hin, hout, geo, jf, x, y, z);
-}
-
-// node i of the list; false past its end.  (Selects over the six segments: an
-// index of f by a runtime value would copy it to local memory; face nodes
-// number fewer than 2^31.)
-__device__ __forceinline__ bool face_coords(const FaceList& f, int i, int& x, int& y, int& z)
-{
-    if (i >= (int)f.start[f.nseg]) return false;
-    int lo0 = 0, lo1 = 0, lo2 = 0, len0 = 1, len1 = 1, st = 0;
-#pragma unroll
-    for (int k = 0; k < 6; k++)
-        if (k < f.nseg && i >= (int)f.start[k]) {
-            lo0 = f.lo[k][0];
-            lo1 = f.lo[k][1];
-            lo2 = f.lo[k][2];
-            len0 = f.len[k][0];
-            len1 = f.len[k][1];
-            st = (int)f.start[k];
-        }
-    const int r = i - st, q = r / len0;
-    x = lo0 + (r - q * len0);
-    y = lo1 + q % len1;
-    z = lo2 + q / len1;
-    return true;
 }
 
 // one step of the face nodes only (the interior comes from the row-staged pass)
@@ -685,19 +729,40 @@ inline void launch_after(void (*kernel)(A...), unsigned grid, unsigned block, cu
     cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-template <class S, class R>
-void launch_momentum(const cslbm_ctx* c, const Lat& L, const S* P, const R* hin, const R* geo)
+// Which lattices take rho u of their face nodes from the boundary rule (one
+// more rounding of numbers that cancel, but the rounding these lattices have
+// always had): FP32 arithmetic, unless AUTO may take the fused pass, which has
+// the closed form; then the gather pass gives the fused pass's bits.  The value
+// of a wall-force objective is a sum of terms hundreds of times larger, so
+// another rounding of the state moves it by several times its error either way
+// (FP32, 22 x 101 x 29, 23 steps from rest: 1.7e-7 with the rule, 5.5e-7 with
+// the closed form; over 16 channels neither is better).
+inline bool momentum_by_rule(const cslbm_ctx* c)
 {
-    const unsigned tb = flat_block(c);
-    launch_after(k_momentum_flat<S, R>, (unsigned)((c->N + tb - 1) / tb), tb, c->stream, L, make_plane(L), P, hin, geo,
-                 (Mom4<R>*)c->jf);
+    return c->p.storage != CSLBM_FP64 && !(c->rows.fused_ok && c->p.step_kernel == CSLBM_STEP_AUTO);
+}
+
+template <class S, class R>
+void launch_momentum(const cslbm_ctx* c, const Lat& L, const S* P, const R* hin, const R* geo, bool rule)
+{
+    const unsigned tb = flat_block(c), nb = (unsigned)((c->N + tb - 1) / tb);
+    if constexpr (!std::is_same<R, double>::value) {
+        const FaceList f = face_list(c);
+        const unsigned nfb = (unsigned)((f.start[f.nseg] + tb - 1) / tb);
+        if (rule && nfb) {
+            launch_after(k_momentum_rule<S, R>, nfb + nb, tb, c->stream, L, make_plane(L), f, nfb, P, hin, geo,
+                         (Mom4<R>*)c->jf);
+            return;
+        }
+    }
+    launch_after(k_momentum_flat<S, R>, nb, tb, c->stream, L, make_plane(L), P, hin, geo, (Mom4<R>*)c->jf);
 }
 
 // one time step: momentum pass, then the step pass
 template <class S, class R>
 void launch_flat_step(const cslbm_ctx* c, const Lat& L, const S* Pin, S* Pout, const R* hin, R* hout, const R* geo)
 {
-    launch_momentum<S, R>(c, L, Pin, hin, geo);
+    launch_momentum<S, R>(c, L, Pin, hin, geo, momentum_by_rule(c));
     const unsigned tb = flat_block(c);
     const FaceList f = face_list(c);
     const unsigned nfb = (unsigned)((f.start[f.nseg] + tb - 1) / tb), n01 = (unsigned)c->n[0] * c->n[1];

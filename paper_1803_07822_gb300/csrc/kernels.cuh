@@ -1007,7 +1007,7 @@ template <class S, class R> struct Launch {
     }
     static void momentum_field(const cslbm_ctx* c)
     {
-        launch_momentum<S, R>(c, make_lat(c), P(c, c->pc), H(c, c->hc), G(c, c->gc));
+        launch_momentum<S, R>(c, make_lat(c), P(c, c->pc), H(c, c->hc), G(c, c->gc), true);
     }
     static int step(cslbm_ctx* c, int mode)
     {

@@ -448,7 +448,7 @@ int launch_rows_step(const cslbm_ctx* c, const Lat& L, int pc, int hc, int gc, i
     const float* hin = (const float*)c->H[hc];
     float* hout = (float*)c->H[1 - hc];
     const float* geo = (const float*)c->G[gc];
-    launch_momentum<S, float>(c, L, Pin, hin, geo);
+    launch_momentum<S, float>(c, L, Pin, hin, geo, momentum_by_rule(c));
     int launched = 1;
     if (pl.ntiles > 0) {
         rows::Maps M;
