@@ -831,6 +831,7 @@ static void interp_corners(const orc_params *p, const double x[3], long idx8[8],
         if (per) {
             xa = fmod(xa, (double)n);
             if (xa < 0) xa += n;
+            if (xa >= n) xa = 0; /* less than half an ulp of n below a period */
         } else {
             if (xa < 0) xa = 0;
             if (xa > n - 1) xa = n - 1;
@@ -838,7 +839,6 @@ static void interp_corners(const orc_params *p, const double x[3], long idx8[8],
         double fl = floor(xa);
         i0[a] = (int)fl;
         t[a] = xa - fl;
-        if (i0[a] >= n) i0[a] = n - 1; /* xa == n after rounding */
         i1[a] = per ? (i0[a] + 1) % n : (i0[a] + 1 < n ? i0[a] + 1 : n - 1);
     }
     for (int c = 0; c < 8; c++) {

@@ -559,6 +559,7 @@ __device__ __forceinline__ void interp_axis(double p, int n, bool per, int& i0, 
     const double dn = (double)n;
     if (per) {
         if (!(p >= 0.0 && p < dn)) p = p < 0.0 && p > -dn ? p + dn : (p >= dn && p < 2.0 * dn ? p - dn : wrap_far(p, n));
+        if (p >= dn) p = 0.0;  // a point less than half an ulp of n below a period
     } else {
         p = fmin(fmax(p, 0.0), (double)(n - 1));
     }
