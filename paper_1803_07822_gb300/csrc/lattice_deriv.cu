@@ -19,7 +19,7 @@
 // sums along one axis that neighbours share, which leaves 10 and 16: blocks
 // march along axis 2 with one plane of a 32 x 8 tile (and its rim) in shared
 // memory, in-plane sums exchanged there, sums along the march kept in
-// registers.  Six fields on 128 x 256 x 128, order 4: 1,359 + 1,150 -> 1,559 us for both.
+// registers.  Six fields on 128 x 256 x 128, order 4: 1,359 + 1,150 -> 1,562 us for both.
 #include <cstdint>
 #include <string>
 
@@ -105,11 +105,6 @@ __device__ __forceinline__ double site(const Box& B, const double* __restrict__ 
     return site_far(B, f, order, x, y, z);
 }
 
-// a site whose whole stencil resolves without continuation (periodic wrap only)
-__device__ __forceinline__ bool inner(const Box& B, int a, int r)
-{
-    return r >= 0 && r < B.n[a] && (r >= 1 || B.plo[a]) && (r <= B.n[a] - 2 || B.phi[a]);
-}
 // The fields and the weights.  The faces of G_i weigh w_1 / c_s^2 = 1/6, its
 // edges w_7 / c_s^2 = 1/12; with order 4 the scratch holds F / 12, so that the
 // gradient below needs no products but by two.
@@ -128,36 +123,17 @@ __global__ void __launch_bounds__(TBL) k_pad(const __grid_constant__ Box B, cons
              (int)(row - zr * ne1) - B.pad[1], (int)zr - B.pad[2]);
 }
 
-// F = f - (c_s^2/2) L f = f0 - sum_l w_l (f_l - f0) at a site whose stencil
-// needs the continuation: with sum_{l>0} w_l = 2/3, w = 1/18 on the six faces,
-// 1/36 on the twelve edges, F = (5/3) f0 - (S_faces + S_edges / 2) / 18
-__device__ __noinline__ double correct_far(const Box& B, const double* __restrict__ f, int x, int y, int z)
-{
-    const double f0 = site(B, f, 4, x, y, z);
-    double sf = 0.0, se = 0.0;
-#pragma unroll 1
-    for (int l = 1; l < Q; l++) {
-        // l = 1..6 faces, 7..18 the edges in the order xy, xz, yz
-        int c[3] = {0, 0, 0};
-        if (l <= 6) {
-            c[(l - 1) >> 1] = l & 1 ? 1 : -1;
-        } else {
-            const int e = (l - 7) >> 2, m = (l - 7) & 3;
-            c[e == 2 ? 1 : 0] = m & 1 ? -1 : 1;
-            c[e == 0 ? 1 : 2] = m & 2 ? -1 : 1;
-        }
-        const double fl = site(B, f, 4, x + c[0], y + c[1], z + c[2]);
-        if (l <= 6) sf += fl;
-        else se += fl;
-    }
-    return fma(5.0 / 3.0, f0, -fma(0.5, se, sf) * (1.0 / 18.0));
-}
-
-// Order 4: F / 12 on the padded lattice.  With the in-plane sums q = s_x + s_y
-// (s_a = f(a + 1) + f(a - 1)) and e = s_x(y + 1) + s_x(y - 1), and u = f + q/2,
+// Order 4: F / 12 on the padded lattice, F = f - (c_s^2/2) L f = f0 - sum_l w_l
+// (f_l - f0) with sum_{l>0} w_l = 2/3, w = 1/18 on the six faces, 1/36 on the
+// twelve edges.  With the in-plane sums q = s_x + s_y (s_a = f(a + 1) + f(a -
+// 1)) and e = s_x(y + 1) + s_x(y - 1), and u = f + q/2,
 //   F = (5/3) f - (q + e/2) / 18 - (u(z + 1) + u(z - 1)) / 18.
-// Planes beyond a face of axis 2 are continued as they are loaded; a site whose
-// stencil leaves the lattice across axis 0 or 1 takes correct_far.
+// Values beyond a face are continued as a plane is loaded, so that every site
+// takes these sums: a constant field's gradient is exactly zero, as for sums
+// written out per site.  (Sites next to a face of axis 0 or 1 in a path of
+// their own, 19 continued sites each, one after the other: 128 x 256 x 128, six
+// fields, both kernels, walls across axis 0 5,553 us against 1,890, across axes
+// 1 and 2 2,628 against 1,599.)
 __global__ void __launch_bounds__(TX* TY) k_correct(const __grid_constant__ Box B, const __grid_constant__ Tiles T,
                                                     const double* __restrict__ f, double* __restrict__ F)
 {
@@ -169,16 +145,31 @@ __global__ void __launch_bounds__(TX* TY) k_correct(const __grid_constant__ Box 
     const double* fc = f + (long long)blockIdx.y * B.N;
     double* Fc = F + (long long)blockIdx.y * B.Ne;
     const bool mine = x < B.n[0] + B.pad[0] && y < B.n[1] + B.pad[1];
-    const bool flat = mine && inner(B, 0, x) && inner(B, 1, y);
-    // the tile's entries this thread loads: in-plane offset, or -1 for none
-    int off[2];
+    // the tile's entries this thread loads: in-plane offset; beyond one face of
+    // the plane that of the face node, with the step inward and the distance
+    // `gone`; kCorner beyond two, kNone for none
+    constexpr int kNone = -1, kCorner = -2;
+    int off[2], step[2], gone[2];
 #pragma unroll
     for (int k = 0; k < 2; k++) {
         const int i = t + k * TX * TY, ly = i / (TX + 2), lx = i - ly * (TX + 2);
         int rx = x0 - 1 + lx, ry = y0 - 1 + ly;
-        off[k] = -1;
-        if (i < (TX + 2) * (TY + 2) && rx <= B.n[0] && ry <= B.n[1] && wrap(B, 0, rx) && wrap(B, 1, ry))
-            off[k] = ry * B.n[0] + rx;
+        off[k] = kNone;
+        step[k] = gone[k] = 0;
+        if (i < (TX + 2) * (TY + 2) && rx <= B.n[0] + B.pad[0] && ry <= B.n[1] + B.pad[1]) {
+            const bool inx = wrap(B, 0, rx), iny = wrap(B, 1, ry);
+            const int r = inx ? ry : rx, n = B.n[inx ? 1 : 0], dir = r < 0 ? 1 : -1;
+            if (!inx && !iny) {
+                off[k] = kCorner;
+            } else {
+                if (!inx || !iny) {
+                    step[k] = dir * (inx ? B.n[0] : 1);
+                    gone[k] = r < 0 ? -r : r - (n - 1);
+                    (inx ? ry : rx) = r < 0 ? 0 : n - 1;
+                }
+                off[k] = ry * B.n[0] + rx;
+            }
+        }
     }
     const unsigned n01 = (unsigned)B.n[0] * B.n[1];
     // u and the in-plane part w of F at plane p (every thread of the block); a
@@ -187,22 +178,24 @@ __global__ void __launch_bounds__(TX* TY) k_correct(const __grid_constant__ Box 
     // face: their rounding is multiplied by the weights.)
     auto plane = [&](int p, double& u, double& w) {
         int pz = p;
-        if (wrap(B, 2, pz)) {
-            const double* fp = fc + (unsigned)pz * n01;
+        const bool in = wrap(B, 2, pz);
+        const double* fp = fc + (in ? (unsigned)pz * n01 : 0u);
 #pragma unroll
-            for (int k = 0; k < 2; k++)
-                if (off[k] >= 0) (&fs[0][0])[t + k * TX * TY] = __ldg(fp + off[k]);
-        } else {
-            const int beyond = p < 0 ? -p : p - (B.n[2] - 1);
+        for (int k = 0; k < 2; k++) {
+            if (off[k] == kNone) continue;
+            const int i = t + k * TX * TY;
+            double v = 0.0;
+            if (off[k] == kCorner || (!in && step[k])) {
+                v = site_far(B, fc, 4, x0 - 1 + i % (TX + 2), y0 - 1 + i / (TX + 2), p);
+            } else if (!in || step[k]) {
+                const int s = in ? step[k] : (p < 0 ? 1 : -1) * (int)n01, g = in ? gone[k] : (p < 0 ? -p : p - (B.n[2] - 1));
+                const double* q = in ? fp + off[k] : fc + (p < 0 ? 0u : (unsigned)(B.n[2] - 1) * n01) + off[k];
 #pragma unroll
-            for (int k = 0; k < 2; k++)
-                if (off[k] >= 0) {
-                    double v = 0.0;
-#pragma unroll
-                    for (int i = 0; i <= 4; i++)
-                        v = fma(cont_weight(4, beyond, i), __ldg(fc + (unsigned)(p < 0 ? i : B.n[2] - 1 - i) * n01 + off[k]), v);
-                    (&fs[0][0])[t + k * TX * TY] = v;
-                }
+                for (int m = 0; m <= 4; m++) v = fma(cont_weight(4, g, m), __ldg(q + (long long)m * s), v);
+            } else {
+                v = __ldg(fp + off[k]);
+            }
+            (&fs[0][0])[i] = v;
         }
         __syncthreads();
         const double sx = fs[ty + 1][tx] + fs[ty + 1][tx + 2];
@@ -220,9 +213,8 @@ __global__ void __launch_bounds__(TX* TY) k_correct(const __grid_constant__ Box 
         plane(p, u, w);
         const int z = p - 1;
         if (p > za && mine) {
-            const double v = flat ? fma(-kEdge / 18.0, ua + u, wb) : kEdge * correct_far(B, fc, x, y, z);
             Fc[((unsigned)(z + B.pad[2]) * B.ne[1] + (unsigned)(y + B.pad[1])) * (unsigned)B.ne[0] +
-               (unsigned)(x + B.pad[0])] = v;
+               (unsigned)(x + B.pad[0])] = fma(-kEdge / 18.0, ua + u, wb);
         }
         ua = ub;
         ub = u;
