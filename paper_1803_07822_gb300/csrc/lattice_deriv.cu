@@ -20,6 +20,8 @@
 // march along axis 2 with one plane of a 32 x 8 tile (and its rim) in shared
 // memory, in-plane sums exchanged there, sums along the march kept in
 // registers.  Six fields on 128 x 256 x 128, order 4: 1,359 + 1,150 -> 1,562 us for both.
+// Lattices that fill the tiles badly keep a thread per site (see
+// gradient_marches).
 #include <cstdint>
 #include <string>
 
@@ -105,6 +107,11 @@ __device__ __forceinline__ double site(const Box& B, const double* __restrict__ 
     return site_far(B, f, order, x, y, z);
 }
 
+// a site whose whole stencil resolves without continuation (periodic wrap only)
+__device__ __forceinline__ bool inner(const Box& B, int a, int r)
+{
+    return r >= 0 && r < B.n[a] && (r >= 1 || B.plo[a]) && (r <= B.n[a] - 2 || B.phi[a]);
+}
 // The fields and the weights.  The faces of G_i weigh w_1 / c_s^2 = 1/6, its
 // edges w_7 / c_s^2 = 1/12; with order 4 the scratch holds F / 12, so that the
 // gradient below needs no products but by two.
@@ -222,6 +229,48 @@ __global__ void __launch_bounds__(TX* TY) k_correct(const __grid_constant__ Box 
     }
 }
 
+// The same per site, for lattices whose tiles would be mostly empty or repeated
+// (correct_marches): 19 loads, those beyond a face one after the other
+__global__ void __launch_bounds__(TBL) k_correct_sites(const __grid_constant__ Box B, const double* __restrict__ f,
+                                                       double* __restrict__ F)
+{
+    const unsigned s = blockIdx.x * TBL + threadIdx.x;
+    if (s >= (unsigned)B.Ne) return;
+    const double* fc = f + (long long)blockIdx.y * B.N;
+    const unsigned ne0 = B.ne[0], ne1 = B.ne[1], row = s / ne0, zr = row / ne1;
+    const int x = (int)(s - row * ne0) - B.pad[0], y = (int)(row - zr * ne1) - B.pad[1], z = (int)zr - B.pad[2];
+    double f0, sf = 0.0, se = 0.0;
+    if (inner(B, 0, x) && inner(B, 1, y) && inner(B, 2, z)) {
+        unsigned o[3][3];
+        const int r[3] = {x, y, z};
+        const unsigned st[3] = {1u, (unsigned)B.n[0], (unsigned)B.n[0] * (unsigned)B.n[1]};
+#pragma unroll
+        for (int a = 0; a < 3; a++)
+#pragma unroll
+            for (int c = -1; c <= 1; c++) {
+                int q = r[a] + c;
+                wrap(B, a, q);
+                o[a][c + 1] = (unsigned)q * st[a];
+            }
+        f0 = __ldg(fc + (o[2][1] + o[1][1] + o[0][1]));
+#pragma unroll
+        for (int l = 1; l < Q; l++) {
+            const double fl = __ldg(fc + (o[2][cvec(l, 2) + 1] + o[1][cvec(l, 1) + 1] + o[0][cvec(l, 0) + 1]));
+            if (l <= 6) sf += fl;
+            else se += fl;
+        }
+    } else {
+        f0 = site(B, fc, 4, x, y, z);
+#pragma unroll
+        for (int l = 1; l < Q; l++) {
+            const double fl = site(B, fc, 4, x + cvec(l, 0), y + cvec(l, 1), z + cvec(l, 2));
+            if (l <= 6) sf += fl;
+            else se += fl;
+        }
+    }
+    F[(long long)blockIdx.y * B.Ne + s] = fma(5.0 / 3.0 * kEdge, f0, (-kEdge / 18.0) * fma(0.5, se, sf));
+}
+
 // d_k f_c = G_k F at every node, out[(k ncomp + c) N + v].  With the
 // differences d_x = F(x + 1) - F(x - 1), d_y, d_z and their sums over the
 // neighbours across,
@@ -306,6 +355,45 @@ __global__ void __launch_bounds__(TX* TY) k_grad(const __grid_constant__ Box B, 
     }
 }
 
+// The same per node, from the nine opposite pairs (gradient_marches)
+template <bool EDGE>
+__global__ void __launch_bounds__(TBL) k_grad_nodes(const __grid_constant__ Box B, int ncomp, const double* __restrict__ F,
+                                                    double* __restrict__ out)
+{
+    const unsigned v = blockIdx.x * TBL + threadIdx.x;
+    if (v >= (unsigned)B.N) return;
+    const int c = blockIdx.y;
+    const double* Fc = F + (long long)c * B.Ne;
+    const unsigned n0 = B.n[0], n1 = B.n[1], row = v / n0, zr = row / n1;
+    // offsets of the sites r + c per axis in the padded lattice
+    unsigned o[3][3];
+    {
+        const int r[3] = {(int)(v - row * n0), (int)(row - zr * n1), (int)zr};
+        const unsigned st[3] = {1u, (unsigned)B.ne[0], (unsigned)B.ne[0] * (unsigned)B.ne[1]};
+#pragma unroll
+        for (int a = 0; a < 3; a++)
+#pragma unroll
+            for (int cc = -1; cc <= 1; cc++) {
+                int q = r[a] + cc;
+                wrap(B, a, q);
+                o[a][cc + 1] = (unsigned)(q + B.pad[a]) * st[a];
+            }
+    }
+    double g[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        const int l = 2 * k + 1;
+        const double d = __ldg(Fc + (o[2][cvec(l, 2) + 1] + o[1][cvec(l, 1) + 1] + o[0][cvec(l, 0) + 1])) -
+                         __ldg(Fc + (o[2][1 - cvec(l, 2)] + o[1][1 - cvec(l, 1)] + o[0][1 - cvec(l, 0)]));
+        const double wd = (l <= 6 ? 2.0 : 1.0) * (EDGE ? kEdge : 1.0);
+#pragma unroll
+        for (int a = 0; a < 3; a++)
+            if (cvec(l, a)) g[a] = fma(cvec(l, a) * wd, d, g[a]);
+    }
+#pragma unroll
+    for (int a = 0; a < 3; a++) out[((long long)a * ncomp + c) * B.N + v] = g[a];
+}
+
 Box box_of(const cslbm_ctx* c, int order)
 {
     Box B;
@@ -350,6 +438,39 @@ size_t pad_bytes(const cslbm_ctx* c, int ncomp, int order)
     return (size_t)ncomp * (size_t)box_of(c, order).Ne * sizeof(double);
 }
 
+// Where the marching kernels pay.  A march takes 0.53 (k_correct), 0.76 (k_grad)
+// or 0.87 (k_grad with the scaling of order 2) of a per-site kernel's time per
+// site it visits, and it visits march_sites: whole tiles, and two planes more
+// per chunk, which are short where the lattice has few tiles.  us, six fields,
+// per-site kernels both / marches both / as chosen here:
+//                        order 2             order 4
+//   48 x 48 x 48          43   61   43        69   82   68   (periodic)
+//   33 x 129 x 65         94  186   94       152  255  153   (periodic)
+//   65 x 129 x 65        183  270  180       291  359  292   (periodic)
+//   64 x 128 x 64        182  193  178       403  248  248   (walls across axis 2)
+//   128 x 256 x 128     1355 1263 1262      2513 1565 1562   (walls across axis 2)
+long long march_sites(const Tiles& T)
+{
+    const int planes = T.last - T.first;
+    return (long long)T.nx * TX * T.ny * TY * (planes + 2 * ((planes + T.chunk - 1) / T.chunk));
+}
+bool gradient_marches(const Tiles& T, const Box& B, int order)
+{
+    return 100 * march_sites(T) <= (order == 2 ? 115 : 130) * B.N;
+}
+// A continued site of k_correct_sites costs 40 others (axes 1 and 2; across
+// axis 0, where every warp has some, several hundred); without faces the march
+// needs 3/4 2^20 sites to fill the device (64 x 128 x 64, one field: 57 us
+// against 55, 96^3: 79 against 85).
+bool correct_marches(const Tiles& T, const Box& B, int ncomp)
+{
+    long long in = 1;
+    for (int a = 0; a < 3; a++) in *= B.n[a] - 2 * B.pad[a];
+    const long long far = B.Ne - in;
+    if (B.pad[0]) return true;
+    return 10 * march_sites(T) <= 17 * B.Ne + 400 * far && (far || B.Ne * ncomp >= 3LL << 18);
+}
+
 cslbm_status gradient(cslbm_ctx* c, const double* f, int ncomp, int order, double* out, void* scratch, size_t bytes)
 {
     if (!c || !f || !out || ncomp < 1 || ncomp > 65535) return lfail(CSLBM_EINVAL, "bad argument");
@@ -360,15 +481,23 @@ cslbm_status gradient(cslbm_ctx* c, const double* f, int ncomp, int order, doubl
         return lfail(CSLBM_EINVAL, "fields, output and scratch must be device memory");
     const Box B = box_of(c, order);
     double* F = (double*)scratch;
-    if (order == 4) {
-        const Tiles T = tiles_of(c->n_sm, B.ne[0], B.ne[1], -B.pad[2], B.n[2] + B.pad[2], ncomp);
-        k_correct<<<tile_grid(T, ncomp), dim3(TX, TY), 0, c->stream>>>(B, T, f, F);
+    const dim3 sites((unsigned)((B.Ne + TBL - 1) / TBL), (unsigned)ncomp);
+    if (order == 2) {
+        k_pad<<<sites, TBL, 0, c->stream>>>(B, f, F);
     } else {
-        k_pad<<<dim3((unsigned)((B.Ne + TBL - 1) / TBL), (unsigned)ncomp), TBL, 0, c->stream>>>(B, f, F);
+        const Tiles T = tiles_of(c->n_sm, B.ne[0], B.ne[1], -B.pad[2], B.n[2] + B.pad[2], ncomp);
+        if (correct_marches(T, B, ncomp)) k_correct<<<tile_grid(T, ncomp), dim3(TX, TY), 0, c->stream>>>(B, T, f, F);
+        else k_correct_sites<<<sites, TBL, 0, c->stream>>>(B, f, F);
     }
     const Tiles T = tiles_of(c->n_sm, B.n[0], B.n[1], 0, B.n[2], ncomp);
-    if (order == 4) k_grad<false><<<tile_grid(T, ncomp), dim3(TX, TY), 0, c->stream>>>(B, T, ncomp, F, out);
-    else k_grad<true><<<tile_grid(T, ncomp), dim3(TX, TY), 0, c->stream>>>(B, T, ncomp, F, out);
+    const dim3 nodes((unsigned)((B.N + TBL - 1) / TBL), (unsigned)ncomp);
+    if (gradient_marches(T, B, order)) {
+        if (order == 4) k_grad<false><<<tile_grid(T, ncomp), dim3(TX, TY), 0, c->stream>>>(B, T, ncomp, F, out);
+        else k_grad<true><<<tile_grid(T, ncomp), dim3(TX, TY), 0, c->stream>>>(B, T, ncomp, F, out);
+    } else {
+        if (order == 4) k_grad_nodes<false><<<nodes, TBL, 0, c->stream>>>(B, ncomp, F, out);
+        else k_grad_nodes<true><<<nodes, TBL, 0, c->stream>>>(B, ncomp, F, out);
+    }
     c->launches += 2;
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return lfail(CSLBM_ECUDA, std::string("lattice gradient: ") + cudaGetErrorString(e));
