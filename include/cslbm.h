@@ -388,7 +388,7 @@ cslbm_status cslbm_batch_step(cslbm_batch* b, int nsteps);
 
 /* Autotuner of the batch step's tile shape: times every candidate -- nodes
  * per block (128, 256, 512) x nodes per work item (1, 4, 16 blocks) x blocks
- * per SM (the resident maximum and half of it) -- on this batch, reps
+ * per SM (the resident maximum, half of it and, of 128 nodes, three) -- on this batch, reps
  * repetitions of one step from the current state each (the state does not
  * advance), keeps the fastest and returns it in shape3 = {nodes per block,
  * nodes per work item, blocks per SM} and its time per step in *ms (either

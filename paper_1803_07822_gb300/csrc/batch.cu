@@ -99,15 +99,48 @@ __device__ __forceinline__ void grid_barrier(unsigned* count, int* err)
     __syncthreads();
 }
 
+// the step of an interior node through registers, nothing staged
+__device__ __forceinline__ void step_plain(const Lat& L, const float* __restrict__ Pin, float* __restrict__ Pout,
+                                           const float* __restrict__ hin, float* __restrict__ hout,
+                                           const float* __restrict__ geo, const Mom4<float>* jf, int x, int y, int z,
+                                           unsigned v)
+{
+    const unsigned N = (unsigned)L.N;
+    const Nbr src = nbr_index(L, x, y, z, -1);
+    float s[Q];
+#pragma unroll
+    for (int l = 0; l < Q; l++)
+        s[l] = Store<float>::ld(Pin + (unsigned)pslot(l) * N + nbr_off(src, cvec(l, 0), cvec(l, 1), cvec(l, 2)));
+    GeoT<float> G;
+    HistT<float> Hp;
+    load_geo_hist(geo, hin, v, N, G, Hp);
+    float d[9][3];
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        // site x + c is the pull source of -c
+        const int l = 2 * k + 1, cx = cvec(l, 0), cy = cvec(l, 1), cz = cvec(l, 2);
+        const Mom4<float> p = jf[nbr_off(src, -cx, -cy, -cz)], m = jf[nbr_off(src, cx, cy, cz)];
+        d[k][0] = p.x - m.x;
+        d[k][1] = p.y - m.y;
+        d[k][2] = p.z - m.z;
+    }
+    step_core<float, float>(L, s, G, Hp, d, Pout, hout, v, N);
+}
+
 // One persistent launch per LBM step of every channel (see the top of the
 // file).  first[c] = first work item of channel c's nodes (items of `item`
 // nodes), first[nchan] = all of them; first[nchan + 1 + c] the same for its
 // face nodes; q the barrier count, zero at launch; k the parity of the step in
 // the two-step cycle.
-template <int TB>
-__global__ void __launch_bounds__(TB, 512 / TB) k_batch_persistent(const Chan* __restrict__ tab,
-                                                                   const unsigned* __restrict__ first, int nchan,
-                                                                   int item, int k, unsigned* q, int* err)
+// STAGED: geometry and history through shared memory (step_interior), 512
+// threads per SM at 128 registers; else step_plain, 384 at 168, which is the
+// faster of the two where the nodes hardly fill one round of blocks (eight
+// channels of 16..40 per side: walls 33 against 31 us per step, periodic 29
+// against 25; 64 channels of 32..96: 1,634 against 1,749).  The tuner picks.
+template <int TB, bool STAGED>
+__global__ void __launch_bounds__(TB, (STAGED ? 512 : 384) / TB)
+    k_batch_persistent(const Chan* __restrict__ tab, const unsigned* __restrict__ first, int nchan, int item, int k,
+                       unsigned* q, int* err)
 {
     extern __shared__ __align__(16) unsigned char smem_batch[];
     float* stage = reinterpret_cast<float*>(smem_batch);
@@ -147,9 +180,12 @@ __global__ void __launch_bounds__(TB, 512 / TB) k_batch_persistent(const Chan* _
         for (unsigned v = v0 + threadIdx.x; v < v1; v += TB) {
             int x, y, z;
             flat_coords(C.L, C.pl, v, x, y, z);
-            if (!on_boundary(C.L, x, y, z))
-                step_interior<float, float, TB, false>(C.L, C.P[pi], C.P[pi ^ 1], C.H[hi], C.H[hi ^ 1], C.G, C.jf, x, y, z, v,
-                                                stage + threadIdx.x);
+            if (on_boundary(C.L, x, y, z)) continue;
+            if constexpr (STAGED)
+                step_interior<float, float, TB, false>(C.L, C.P[pi], C.P[pi ^ 1], C.H[hi], C.H[hi ^ 1], C.G, C.jf, x, y, z,
+                                                       v, stage + threadIdx.x);
+            else
+                step_plain(C.L, C.P[pi], C.P[pi ^ 1], C.H[hi], C.H[hi ^ 1], C.G, C.jf, x, y, z, v);
         }
     }
 }
@@ -167,7 +203,7 @@ using cslbm::batch::Chan;
 struct Shape {
     int tb;    // index into kTB
     int item;  // nodes per work item
-    int bps;   // blocks per SM
+    int bps;   // blocks per SM; with 128 threads three are those of the kernel that stages nothing
 };
 
 struct cslbm_batch {
@@ -247,7 +283,7 @@ cslbm_status upload_table(cslbm_batch* b)
     return CSLBM_OK;
 }
 
-template <int TB>
+template <int TB, bool STAGED = true>
 cudaError_t launch_tb(cslbm_batch* b, const Shape& sh, int k, cudaStream_t s)
 {
     const unsigned* first = b->d_first + item_index(sh.item) * 2 * (b->nb + 1);
@@ -261,8 +297,8 @@ cudaError_t launch_tb(cslbm_batch* b, const Shape& sh, int k, cudaStream_t s)
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, cslbm::batch::k_batch_persistent<TB>, (const Chan*)b->d_tab, first, b->nb,
-                              sh.item, k, b->d_q, b->d_err);
+    return cudaLaunchKernelEx(&cfg, cslbm::batch::k_batch_persistent<TB, STAGED>, (const Chan*)b->d_tab, first,
+                              b->nb, sh.item, k, b->d_q, b->d_err);
 }
 
 // one LBM step of every channel: the barrier reset, then one persistent launch
@@ -271,29 +307,34 @@ cudaError_t launch_step(cslbm_batch* b, const Shape& sh, int k, cudaStream_t s)
     cudaError_t e = cudaMemsetAsync(b->d_q, 0, 4 * sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     switch (sh.tb) {
-    case 0: return launch_tb<128>(b, sh, k, s);
+    case 0: return sh.bps == 3 ? launch_tb<128, false>(b, sh, k, s) : launch_tb<128>(b, sh, k, s);
     case 1: return launch_tb<256>(b, sh, k, s);
     default: return launch_tb<512>(b, sh, k, s);
     }
 }
 
-template <int TB> int occupancy_tb(const cslbm_batch* b)
+template <int TB, bool STAGED> int occupancy_tb(const cslbm_batch* b)
 {
-    const size_t sm = cslbm::batch::smem_bytes<TB>(b->nb);
     // (the most channels a batch can have, so that the attribute serves every batch)
-    cslbm::set_smem_optin_once<cslbm::batch::k_batch_persistent<TB>>(
+    cslbm::set_smem_optin_once<cslbm::batch::k_batch_persistent<TB, STAGED>>(
         b->ctx[0]->device, (int)cslbm::batch::smem_bytes<TB>(cslbm::batch::kMaxChan));
     int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cslbm::batch::k_batch_persistent<TB>, TB, sm);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cslbm::batch::k_batch_persistent<TB, STAGED>, TB,
+                                                  cslbm::batch::smem_bytes<TB>(b->nb));
     return occ;
 }
 int occupancy(const cslbm_batch* b, int tb)
 {
     switch (tb) {
-    case 0: return occupancy_tb<128>(b);
-    case 1: return occupancy_tb<256>(b);
-    default: return occupancy_tb<512>(b);
+    case 0: return occupancy_tb<128, true>(b);
+    case 1: return occupancy_tb<256, true>(b);
+    default: return occupancy_tb<512, true>(b);
     }
+}
+// may the batch launch with this shape's block size and blocks per SM?
+bool resident(const cslbm_batch* b, int tb, int bps)
+{
+    return bps >= 1 && bps <= occupancy(b, tb) && (tb != 0 || bps != 3 || occupancy_tb<128, false>(b) >= 3);
 }
 
 cslbm_status make_graph(cslbm_batch* b)
@@ -387,6 +428,11 @@ cslbm_status cslbm_batch_create(int nb, const cslbm_params* p, void* workspace, 
         const int occ = occupancy(b, 1);
         if (occ < 1) st = bfail(CSLBM_ECUDA, "the batch kernel cannot be resident");
         else b->shape.bps = occ;
+        // (an untuned batch that would leave blocks without an item: two periodic
+        // channels of 16..24 per side 31 -> 15 us per step)
+        long long nodes = 0;
+        for (const cslbm_ctx* c : b->ctx) nodes += c->N;
+        if (nodes < 1024LL * occ * b->n_sm) b->shape.item = 256;
     }
     if (!st) {
         if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess)
@@ -462,16 +508,16 @@ cslbm_status cslbm_batch_tune(cslbm_batch* b, int reps, int* shape3, float* ms)
     if (!table_current(b))
         if (cslbm_status s = upload_table(b)) return s;
     // candidates: block size x work-item size x blocks per SM (the resident
-    // maximum and half of it); the same step (parity 0) repeated, so every
+    // maximum, half of it, and three of 128 threads); the same step (parity 0) repeated, so every
     // repetition reads the current state and writes the spare buffers
     b->cand.clear();
     b->cand_ms.clear();
     for (int t = 0; t < 3; t++) {
         const int occ = occupancy(b, t);
         if (occ < 1) continue;
-        const int bps_c[2] = {occ, occ / 2};
-        for (int u = 0; u < 2; u++) {
-            if (bps_c[u] < 1 || (u == 1 && bps_c[1] == bps_c[0])) continue;
+        const int bps_c[3] = {occ, occ / 2, t == 0 ? 3 : 0};
+        for (int u = 0; u < 3; u++) {
+            if (!resident(b, t, bps_c[u]) || (u && bps_c[u] == occ)) continue;
             for (int mi = 0; mi < 3; mi++) b->cand.push_back({t, cslbm::batch::kTB[t] * cslbm::batch::kItemMul[mi], bps_c[u]});
         }
     }
@@ -512,7 +558,7 @@ cslbm_status cslbm_batch_set_shape(cslbm_batch* b, const int* shape3)
     bool item_ok = false;
     for (int k = 0; k < 7; k++)
         if (cslbm::batch::kItems[k] == shape3[1]) item_ok = true;
-    if (t < 0 || !item_ok || shape3[1] % shape3[0] != 0 || shape3[2] < 1 || shape3[2] > occupancy(b, t))
+    if (t < 0 || !item_ok || shape3[1] % shape3[0] != 0 || !resident(b, t, shape3[2]))
         return bfail(CSLBM_EINVAL, "nodes per block 128, 256 or 512; nodes per work item a multiple of it in "
                                    "128..8192 (powers of two); blocks per SM from 1 to the resident maximum");
     b->shape = {t, shape3[1], shape3[2]};
