@@ -559,14 +559,13 @@ __device__ __forceinline__ void interp_axis(double p, int n, bool per, int& i0, 
     const double dn = (double)n;
     if (per) {
         if (!(p >= 0.0 && p < dn)) p = p < 0.0 && p > -dn ? p + dn : (p >= dn && p < 2.0 * dn ? p - dn : wrap_far(p, n));
-        if (p >= dn) p = 0.0;  // a point less than half an ulp of n below a period
     } else {
         p = fmin(fmax(p, 0.0), (double)(n - 1));
     }
     const double fl = floor(p);
     i0 = (int)fl;
     t = p - fl;
-    if (i0 >= n) i0 = n - 1;
+    if (i0 >= n) i0 = 0;  // a point less than half an ulp of n below a period: p = n, the first node
     i1 = per ? (i0 + 1 == n ? 0 : i0 + 1) : (i0 + 1 < n ? i0 + 1 : n - 1);
 }
 
