@@ -893,8 +893,12 @@ __global__ void __launch_bounds__(TB, sizeof(R) == 8 ? 2 : 5) k2_readout(const _
     bool odd = sizeof(R) == 8;
     if constexpr (sizeof(R) == 4) {
         const double ir = cslbm::recip64(rho, r, odd);
-        u0 = cslbm::widen(j[0], odd) * ir;
-        u1 = cslbm::widen(j[1], odd) * ir;
+        // (one residual correction: the rounded quotient, as a division gives it)
+        const double j0 = cslbm::widen(j[0], odd), j1 = cslbm::widen(j[1], odd);
+        u0 = j0 * ir;
+        u1 = j1 * ir;
+        u0 = fma(fma(-u0, r, j0), ir, u0);
+        u1 = fma(fma(-u1, r, j1), ir, u1);
     }
     if (odd) {
         r = double(rho);
