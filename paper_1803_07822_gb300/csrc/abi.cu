@@ -4,7 +4,6 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
-#include <mutex>
 #include <string>
 
 #include "ctx.h"
@@ -180,60 +179,49 @@ cslbm_status read_scratch(cslbm_ctx* c, double* out, int k)
     return CSLBM_OK;
 }
 
-// Mapped host memory the reductions write their result to: 64 slots of four
-// doubles in one page of the process, taken by a context's first reduction and
-// given back by cslbm_destroy (a context without one copies its result).
-constexpr int kSlots = 64;
-std::mutex g_slot_mu;
-double* g_slot_page = nullptr;
-unsigned long long g_slot_used = 0;
-
-double* slot_take()
-{
-    std::lock_guard<std::mutex> lock(g_slot_mu);
-    if (!g_slot_page) {
+// the reductions' mapped host memory (a context without a slot copies its result)
+struct Mapped {
+    static double* alloc()
+    {
         // (another thread may be capturing a stream)
         cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
         cudaThreadExchangeStreamCaptureMode(&mode);
         void* p = nullptr;
         void* d = nullptr;
-        if (cudaHostAlloc(&p, kSlots * 4 * sizeof(double), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess) {
-            if (cudaHostGetDevicePointer(&d, p, 0) == cudaSuccess && d == p) g_slot_page = (double*)p;
-            else cudaFreeHost(p);
+        if (cudaHostAlloc(&p, 64 * 4 * sizeof(double), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) p = nullptr;
+        else if (cudaHostGetDevicePointer(&d, p, 0) != cudaSuccess || d != p) {
+            cudaFreeHost(p);
+            p = nullptr;
         }
         cudaThreadExchangeStreamCaptureMode(&mode);
         cudaGetLastError();
-        if (!g_slot_page) return nullptr;
+        return (double*)p;
     }
-    for (int i = 0; i < kSlots; i++)
-        if (!(g_slot_used >> i & 1)) {
-            g_slot_used |= 1ull << i;
-            return g_slot_page + 4 * i;
-        }
-    return nullptr;
-}
-void slot_give(double* s)
-{
-    if (!s) return;
-    std::lock_guard<std::mutex> lock(g_slot_mu);
-    g_slot_used &= ~(1ull << ((s - g_slot_page) / 4));
-}
+    static bool alive(const double* page)
+    {
+        cudaPointerAttributes at;
+        const bool ok = cudaPointerGetAttributes(&at, page) == cudaSuccess && at.type == cudaMemoryTypeHost;
+        cudaGetLastError();
+        return ok;
+    }
+};
+cslbm::SlotPool<Mapped> g_slots;
 
 // k sums of a reduction launched by run(acc, host): through the context's
 // slot, else through the scratch with a copy
 template <class F> cslbm_status reduce(cslbm_ctx* c, double* out, int k, const char* what, F run)
 {
     if (!c->slot_tried) {
-        c->slot = slot_take();
+        c->slot = g_slots.take();
         c->slot_tried = 1;
     }
     double* acc = c->scratch + 8;  // zero between reductions
-    run(acc, c->slot);
+    run(acc, c->slot.p);
     c->launches++;
     LAUNCH_CHECK(what);
-    if (c->slot) {
+    if (c->slot.p) {
         CUDA_TRY(cudaStreamSynchronize(c->stream));
-        for (int i = 0; i < k; i++) out[i] = ((volatile double*)c->slot)[i];
+        for (int i = 0; i < k; i++) out[i] = ((volatile double*)c->slot.p)[i];
         return CSLBM_OK;
     }
     CUDA_TRY(cudaMemcpyAsync(out, acc, k * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
@@ -413,7 +401,7 @@ cslbm_status cslbm_create(const cslbm_params* p, void* ws, size_t bytes, void* s
         c->face_n[k] = L.face_n[k];
     }
     c->scratch = (double*)(b + L.off_scratch);
-    c->slot = nullptr;
+    c->slot = {};
     c->slot_tried = 0;
     c->rows.done = (unsigned*)(b + L.off_done);
     c->staging = (double*)(b + L.off_staging);
@@ -446,7 +434,7 @@ cslbm_status cslbm_destroy(cslbm_ctx* c)
     if (!c) return fail(CSLBM_EINVAL, "ctx is null");
     cudaStreamSynchronize(c->stream);
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
-    slot_give(c->slot);
+    g_slots.give(c->slot);
     delete c;
     return CSLBM_OK;
 }

@@ -10,6 +10,7 @@
 
 #include "../../include/cslbm.h"
 #include "rows_plan.h"
+#include "slots.h"
 
 struct cslbm_ops;
 
@@ -55,7 +56,7 @@ struct cslbm_ctx {
     double* face[6]; // [3][face nodes] boundary velocity of non-periodic faces
     long long face_n[6];
     double* scratch; // 64 doubles of reduction space
-    double* slot;    // four doubles of mapped host memory for reduced values, or null
+    cslbm::Slot slot;  // mapped host memory for reduced values, or none
     int slot_tried;
     double* staging; // host-transfer staging, chunk * 24 doubles
     long long chunk; // nodes per staging chunk
