@@ -423,16 +423,6 @@ cslbm_status check_order(const cslbm_ctx* c, int order)
     return CSLBM_OK;
 }
 
-bool device_memory(const void* p)
-{
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
-}
-
 size_t pad_bytes(const cslbm_ctx* c, int ncomp, int order)
 {
     return (size_t)ncomp * (size_t)box_of(c, order).Ne * sizeof(double);
@@ -477,7 +467,7 @@ cslbm_status gradient(cslbm_ctx* c, const double* f, int ncomp, int order, doubl
     if (cslbm_status s = check_order(c, order)) return s;
     const size_t need = pad_bytes(c, ncomp, order);
     if (!scratch || bytes < need) return lfail(CSLBM_ENOMEM, "scratch smaller than required");
-    if (!device_memory(f) || !device_memory(out) || !device_memory(scratch))
+    if (!cslbm_is_device_memory(f) || !cslbm_is_device_memory(out) || !cslbm_is_device_memory(scratch))
         return lfail(CSLBM_EINVAL, "fields, output and scratch must be device memory");
     const Box B = box_of(c, order);
     double* F = (double*)scratch;
@@ -550,7 +540,7 @@ cslbm_status cslbm_update_metric_lattice(cslbm_ctx* c, const double* g6, const d
     size_t need = 0;
     if (cslbm_status s = cslbm_metric_lattice_scratch_bytes(c, order, &need)) return s;
     if (!g6 || !Jnew9 || !scratch || scratch_bytes < need) return lfail(CSLBM_ENOMEM, "scratch smaller than required");
-    if (!device_memory(Jnew9)) return lfail(CSLBM_EINVAL, "Jnew9 must be device memory");
+    if (!cslbm_is_device_memory(Jnew9)) return lfail(CSLBM_EINVAL, "Jnew9 must be device memory");
     double* dg = (double*)scratch;
     const size_t dg_bytes = 18 * (size_t)c->N * sizeof(double);
     if (cslbm_status s = gradient(c, g6, 6, order, dg, (char*)scratch + dg_bytes, scratch_bytes - dg_bytes)) return s;

@@ -1,8 +1,5 @@
-// Arithmetic of one LBM step written for a value type T that is either one
-// node's scalar (float / double) or a pair of x-adjacent nodes (Pair<float>,
-// Pair<double>).  For Pair<float> every operation is one packed FP32
-// instruction (FADD2 / FMUL2 / FFMA2), so a thread steps two nodes for the
-// instruction count of one.
+// Arithmetic of one LBM step of one node, T its scalar (float or double), in
+// explicit fused multiply-adds, so that every pass gives the same bits.
 //
 // The D3Q19 populations come in opposite pairs (l, l+1) for odd l, which the
 // sums and the Hermite recomposition exploit: with p = s_l + s_l+1 and
@@ -14,46 +11,6 @@
 #include "lbm_device.cuh"
 
 namespace cslbm {
-
-template <class R> struct Pair;
-
-template <> struct Pair<float> {
-    float2 v;
-    __device__ __forceinline__ Pair() {}
-    __device__ __forceinline__ Pair(float a) : v(make_float2(a, a)) {}
-    __device__ __forceinline__ Pair(float a, float b) : v(make_float2(a, b)) {}
-    __device__ __forceinline__ explicit Pair(float2 x) : v(x) {}
-    __device__ __forceinline__ float lo() const { return v.x; }
-    __device__ __forceinline__ float hi() const { return v.y; }
-};
-__device__ __forceinline__ Pair<float> operator+(Pair<float> a, Pair<float> b) { return Pair<float>(__fadd2_rn(a.v, b.v)); }
-__device__ __forceinline__ Pair<float> operator-(Pair<float> a, Pair<float> b)
-{
-    return Pair<float>(__fadd2_rn(a.v, make_float2(-b.v.x, -b.v.y)));
-}
-__device__ __forceinline__ Pair<float> operator*(Pair<float> a, Pair<float> b) { return Pair<float>(__fmul2_rn(a.v, b.v)); }
-__device__ __forceinline__ Pair<float> fmad(Pair<float> a, Pair<float> b, Pair<float> c)
-{
-    return Pair<float>(__ffma2_rn(a.v, b.v, c.v));
-}
-__device__ __forceinline__ Pair<float> recip(Pair<float> a) { return Pair<float>(1.0f / a.v.x, 1.0f / a.v.y); }
-
-template <> struct Pair<double> {
-    double x, y;
-    __device__ __forceinline__ Pair() {}
-    __device__ __forceinline__ Pair(double a) : x(a), y(a) {}
-    __device__ __forceinline__ Pair(double a, double b) : x(a), y(b) {}
-    __device__ __forceinline__ double lo() const { return x; }
-    __device__ __forceinline__ double hi() const { return y; }
-};
-__device__ __forceinline__ Pair<double> operator+(Pair<double> a, Pair<double> b) { return Pair<double>(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ Pair<double> operator-(Pair<double> a, Pair<double> b) { return Pair<double>(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ Pair<double> operator*(Pair<double> a, Pair<double> b) { return Pair<double>(a.x * b.x, a.y * b.y); }
-__device__ __forceinline__ Pair<double> fmad(Pair<double> a, Pair<double> b, Pair<double> c)
-{
-    return Pair<double>(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
-}
-__device__ __forceinline__ Pair<double> recip(Pair<double> a) { return Pair<double>(1.0 / a.x, 1.0 / a.y); }
 
 __device__ __forceinline__ float fmad(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fmad(double a, double b, double c) { return fma(a, b, c); }
