@@ -448,7 +448,7 @@ cslbm_status cslbm_batch_create(int nb, const cslbm_params* p, void* workspace, 
                                b->stream) != cudaSuccess)
         st = bfail(CSLBM_ECUDA, "table upload failed");
     if (!st && cudaMemsetAsync(b->d_q, 0, 4 * sizeof(unsigned) + sizeof(int), b->stream) != cudaSuccess)
-        st = bfail(CSLBM_ECUDA, "queue reset failed");
+        st = bfail(CSLBM_ECUDA, "barrier reset failed");
     if (!st && cudaStreamSynchronize(b->stream) != cudaSuccess) st = bfail(CSLBM_ECUDA, "table upload failed");
     if (st) {
         if (have_stream) cudaStreamDestroy(b->stream);

@@ -17,7 +17,8 @@
 // populations and the stencil load (64x128x64: 76.6 -> 46 us per step, 91 x
 // 77 x 93: 94 -> 60, 256^3: 1,717 -> 1,334 with the following), face nodes
 // run in blocks of their own ahead of the others instead of on a slow branch
-// of every warp, rho u of a face node needs no boundary rule, blocks shrink
+// of every warp (rho u of a face node in closed form where that keeps the bits,
+// momentum_by_rule), blocks shrink
 // until every SM has four (16 x 32 x 16: 22.6 -> 13.3 us per step, FP64 106
 // -> 51), and each kernel's blocks come up while the previous one drains.
 // Measured without effect: five blocks per SM, blocks of 64 or 160 nodes,

@@ -63,10 +63,15 @@ inline bool make_plan(const int n[3], bool yper, bool zper, int s_bytes, int max
 }
 
 // The pass AUTO takes where the row passes apply.  They need full tiles (TR n0 =
-// NT: all compute threads busy, grouped copies; 192-node rows: 742 us fused,
-// 574 gather at 192^3 FP32) of one or two rows (four rows of 64: 103 rows, 87
-// gather at 64x128x128) and enough nodes to fill the copy pipeline; the
-// fused form pays its waits back only well beyond L2.  us per step:
+// NT: all compute threads busy, grouped copies) of one or two rows and enough
+// nodes to fill the copy pipeline; the fused form pays its waits back only well
+// beyond L2.  All passes give the same bits.  us per step, FP32, walls across
+// axis 2, n0 x 256 x 256:
+//     n0     32   48   64   96  100  128  160  192   208   224   240   252   256
+//   gather  167  251  329  496  517  654  825  989  1075  1154  1241  1294  1307
+//   rows    229  290  333  583  610  604 1059 1132  1198  1238  1317  1409  1164
+//   fused   236  300  349  637  647  593 1241 1254  1276  1285  1256  1296  1102
+// and across the lines:
 //   FP32, walls across axis 2    gather  rows  fused   | periodic  gather  rows
 //     256x256x16   (1.0 M)         93     95    112    |             86     78
 //     256x256x32   (2.1 M)        174    168    181    |            167    153

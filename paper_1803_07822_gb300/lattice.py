@@ -33,8 +33,9 @@ class CurvedLattice:
     tau: BGK relaxation time; fext: contravariant body-force density;
     storage: "fp32", "fp16", "bf16" (weight-shifted, FP32 arithmetic) or
     "fp64"; literal_a2: transform a_(2) itself on chart changes;
-    step_kernel: "auto" (fused row pass, else row pass, else flat pass),
-    "rows" (row pass with a separate momentum kernel) or "flat".
+    step_kernel: "auto" (the fused row pass, the row pass or the flat gather
+    pass by size, cslbm.h), "rows" (row pass with a separate momentum kernel
+    where it applies) or "flat".
     """
 
     def __init__(self, n, bc_lo=(0, 0, 0), bc_hi=None, tau=0.8, theta=0.0, fext=(0.0, 0.0, 0.0),
