@@ -239,9 +239,13 @@ __device__ __forceinline__ bool face_coords(const FaceList& f, int i, int& x, in
 }
 
 // The same with the boundary rule on face nodes (momentum_by_rule), which the
-// first nfb blocks take: 91 x 77 x 93 FP32, ten steps and the fields, 654 -> 659 us
-template <class S, class R>
-__global__ void __launch_bounds__(FB)
+// first nfb blocks take.  MINB: eight blocks per SM (64 registers, the rule
+// spills 48 bytes) where the memory bounds the pass, one (80 registers) where
+// the rule's chain of loads does (us per step, closed form / one / eight: 21 x
+// 33 x 17 8.9, 9.5, 10.3; 91 x 77 x 93 55.0, 55.3, 54.8; 257 x 128 x 128 334,
+// 341, 336).
+template <class S, class R, int MINB>
+__global__ void __launch_bounds__(FB, MINB)
     k_momentum_rule(const __grid_constant__ Lat L, const __grid_constant__ Plane pl, const __grid_constant__ FaceList f,
                     unsigned nfb, const S* __restrict__ P, const R* __restrict__ hist, const R* __restrict__ geo,
                     Mom4<R>* __restrict__ jf)
@@ -751,8 +755,8 @@ void launch_momentum(const cslbm_ctx* c, const Lat& L, const S* P, const R* hin,
         const FaceList f = face_list(c);
         const unsigned nfb = (unsigned)((f.start[f.nseg] + tb - 1) / tb);
         if (rule && nfb) {
-            launch_after(k_momentum_rule<S, R>, nfb + nb, tb, c->stream, L, make_plane(L), f, nfb, P, hin, geo,
-                         (Mom4<R>*)c->jf);
+            launch_after(tb < FB ? k_momentum_rule<S, R, 1> : k_momentum_rule<S, R, 8>, nfb + nb, tb, c->stream, L,
+                         make_plane(L), f, nfb, P, hin, geo, (Mom4<R>*)c->jf);
             return;
         }
     }
