@@ -797,21 +797,29 @@ __device__ __forceinline__ double density_velocity(double rho, const double j[3]
     return rho;
 }
 
+// Threads of a readout block.  FP64 in small ones, taken from both ends of the
+// nodes inwards, with the boundary rule in line at 128 registers: face nodes take
+// several times an interior node's time, and a block waits for them, the last
+// ones longest (out of line at 64 registers the rule spilled 680 bytes).
+// Contravariant, us, three divisions per node / now: 12 x 10 x 9 walls across every
+// axis 33 / 17, 60^3 walls across axis 1 65 / 64, 100 x 75 x 50 inflow, outflow and
+// walls 108 / 97, 128^3 walls across axis 2 441 / 387, across every axis 1,081 / 992.
+template <class R> constexpr int kReadout = sizeof(R) == 8 ? 64 : TPB;
+
 template <class S, class R>
-__global__ void __launch_bounds__(TPB, sizeof(R) == 8 ? 2 : 4) k_readout(const __grid_constant__ Lat L, const S* __restrict__ P, const R* __restrict__ hist,
+__global__ void __launch_bounds__(kReadout<R>, sizeof(R) == 8 ? 8 : 4) k_readout(const __grid_constant__ Lat L, const S* __restrict__ P, const R* __restrict__ hist,
                                                  const R* __restrict__ geo, const R* __restrict__ J,
                                                  double* __restrict__ rho_out, double* __restrict__ u_out,
                                                  long long stride, long long v0, long long cnt, int cartesian)
 {
-    long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const unsigned blk = sizeof(R) == 8 ? (blockIdx.x & 1 ? gridDim.x - 1 - (blockIdx.x >> 1) : blockIdx.x >> 1) : blockIdx.x;
+    const long long t = blk * (long long)blockDim.x + threadIdx.x;
     if (t >= cnt) return;
     long long v = v0 + t;
     int x, y, z;
     node_coords(L, v, x, y, z);
     R rho, j[3];
     if constexpr (sizeof(R) == 8) {
-        // (the boundary rule in line at 128 registers: out of line at 64 it spilled, walls
-        // across every axis contravariant 128^3 1,124 us, 1,082 with three divisions, now 997)
         NodeMoments<S, R> M;
         node_moments<S, R>(L, P, hist, geo, x, y, z, v, geo[v], M);
         rho = M.rho;
@@ -1081,7 +1089,7 @@ template <class S, class R> struct Launch {
     static void readout(const cslbm_ctx* c, double* rho, double* u3, long long stride, long long v0, long long cnt,
                         int cartesian)
     {
-        k_readout<S, R><<<nblocks(cnt), TPB, 0, c->stream>>>(make_lat(c), P(c, c->pc), H(c, c->hc), G(c, c->gc), (const R*)c->J,
+        k_readout<S, R><<<(unsigned)((cnt + kReadout<R> - 1) / kReadout<R>), kReadout<R>, 0, c->stream>>>(make_lat(c), P(c, c->pc), H(c, c->hc), G(c, c->gc), (const R*)c->J,
                                                              rho, u3, stride, v0, cnt, cartesian);
     }
     static void mass(const cslbm_ctx* c, double* acc, double* host)
